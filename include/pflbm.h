@@ -99,7 +99,13 @@ typedef struct {
     /* Step kernel (results are identical bit for bit; only the speed
      * differs). 0: the library's default, by the measured crossover: 4 for
      * 16-bit storage on lattices of at least 2^19 nodes and for FP32 on
-     * lattices of at least 2^21 nodes, else 1;
+     * lattices of at least 2^21 nodes, else 1; runs of at least 16 steps
+     * of a lattice that fits the chip's shared memory (up to about 270,000
+     * fluid nodes in FP32, 310,000 in 16-bit storage, 75,000 in FP64) are
+     * then taken many steps per launch, the lattice held there (they
+     * allocate exchange memory on first use, beyond
+     * pflbm_footprint_bytes; without it, and on a stream under capture,
+     * the steps run one launch each);
      * 1: populations pulled from global memory, 32 x 8 tiles; 2:
      * populations staged in shared memory by TMA, 32 x 8 tiles; 3: staged,
      * 64 x 4 tiles; 4: global loads, two x-adjacent nodes per thread in

@@ -123,6 +123,39 @@ struct Params {           // derived parameters (Sec. 2.1-2.2), in FP64
 
 struct TmaSet;            // tensor maps of the staged step (step_core.cuh)
 
+// How a lattice is cut for the steps that hold it in shared memory
+// (resident.cu): px x py patches, those with a zeta = 1 node active.
+constexpr int kMaxPatches = 1024;
+struct ResidentCut {
+    int px, py;
+    int units, rows;                    // columns / nodes per lane (rounded up), ny - 2
+    int max_slots;                      // exchange words per type and patch
+    uint32_t active[kMaxPatches / 32];
+};
+struct ResidentPlan {
+    ResidentCut cut{};
+    int cls = 0, nt = 0, n_active = 0;  // patch class, threads per CTA, CTAs
+    unsigned long long words = 0;       // exchange words (both buffers)
+    size_t bytes = 0;                   // the words and the lists' overflow
+};
+// 8 x 8 blocks with a fluid node, as a summed-area table.
+struct SolidMap {
+    int bw = 0, bh = 0;
+    std::vector<int> sum;
+    void build(const uint8_t* solid, int nx, int ny);
+};
+// One launch over patches of several lattices.
+struct ResidentWave {
+    const void* args;                   // step descriptors (device)
+    const ResidentCut* cuts;
+    const uint4* items;                 // member, patch, first word (64 bits)
+    void* words;
+    unsigned long long half;
+    uint32_t* spill;
+    unsigned tag;
+    int steps, n_items;
+};
+
 }  // namespace pfk
 
 // The handle.
@@ -172,6 +205,13 @@ struct pflbm {
     int step_shape = -1;          // -1: global-load step kernel; 0: 32 x 8; 1: 64 x 4 staged;
                                   // -2: global loads, two nodes per thread (packed FP32x2)
     int step_chunk = 16;          // staged step: tiles per work item (blocks a CTA marches)
+    // resident steps (resident.cu): plan and exchange words, made on first use
+    pfk::SolidMap map;            // lattices small enough for it only
+    bool auto_kernel = true;      // the step kernel is the library's choice
+    int res_state = 0;            // 0: not tried, 1: ready, -1: not for this lattice
+    pfk::ResidentPlan res;
+    void* res_words = nullptr;
+    unsigned res_tag = 0;         // tag of the last exchange
 };
 
 namespace pfk {
@@ -200,6 +240,16 @@ __host__ __device__ inline int tiles_y(int ny) { return (ny + TY - 1) / TY; }
 cudaError_t launch_init_phi_droplet(pflbm_t* h, double x0, double y0, double R, int replace);
 cudaError_t launch_init_populations(pflbm_t* h);
 cudaError_t launch_step(pflbm_t* h);
+// resident.cu: many steps in one cooperative launch, the lattice in shared memory
+// (only_class < 0: any patch class)
+bool plan_resident(int nx, int ny, int precision, const SolidMap& map, int max_ctas, int only_class,
+                   ResidentPlan* out);
+size_t resident_word_bytes();
+int resident_batch_class(int precision);              // patch class of batches; < 0: none
+int resident_spill(int precision, int cls);           // 32-bit words of list overflow per CTA
+cudaError_t launch_resident_wave(int precision, const ResidentWave& w, int cls, cudaStream_t stream);
+cudaError_t launch_resident(pflbm_t* h, const ResidentPlan& plan, int steps);
+unsigned bounds_violations_resident();
 // step2.cu: two x-adjacent nodes per thread in packed FP32x2 (FP32, 16-bit)
 cudaError_t launch_step2(pflbm_t* h);
 size_t node_words_bytes(int nx, int ny);
