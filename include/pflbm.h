@@ -271,8 +271,11 @@ typedef struct {
                             arithmetic), one launch per group of lattices
                             of one size, one 64 x 8 tile per CTA, the
                             groups' launches side by side (tiles_per_item,
-                            order and ctas_per_sm do not apply). FP64
-                            batches always use 1.                           */
+                            order and ctas_per_sm do not apply). Runs of at
+                            least 16 steps take the members that fit the
+                            chip's shared memory many steps per launch
+                            instead (16-bit storage, and FP32 batches of up
+                            to 2^21 nodes). FP64 batches always use 1.      */
     /* Staged kernel, per size class: a lattice with nx * ny <=
      * class_max_nodes[k] (first such k < n_classes) runs with tile shape
      * class_shape[k] (0: 32 x 8, 1: 64 x 4) and class_tiles[k] tiles per

@@ -12,6 +12,10 @@
 // joined back. With use_graph the launches of PFLBM_BATCH_GRAPH_STEPS steps
 // are captured once in a CUDA graph and replayed; in it each group takes its
 // steps back to back on its stream, and the streams join once per replay.
+//
+// Runs of 16 steps and more with schedule kernel 3 or 0 step the members that
+// fit the chip's shared memory there, many steps per launch (resident.cu), in
+// waves of as many members as it holds; the rest of the batch as above.
 #include <algorithm>
 #include <climits>
 #include <cstring>
@@ -46,6 +50,19 @@ struct pflbm_batch {
         std::vector<unsigned char> descs[2];   // count step descriptors of each set (host)
     };
     std::vector<ClassLaunch> classes;
+    // runs of many steps: members that fit the chip's shared memory are stepped
+    // there (resident.cu), as many of them side by side as it holds (a wave),
+    // wave by wave; the others as above (their own groups and graph)
+    struct Wave { int first, count; };     // its items
+    std::vector<Wave> waves;
+    std::vector<ClassLaunch> rest;
+    uint4* d_items = nullptr;
+    ResidentCut* d_cuts = nullptr;
+    void* d_words = nullptr;
+    size_t cap_items = 0, cap_cuts = 0, cap_words = 0;   // bytes
+    unsigned long long half_words = 0;     // exchange words of one buffer
+    size_t spill_at = 0;                   // byte offset of the lists' overflow in d_words
+    unsigned res_tag = 0;
     // per-class launches run side by side: forked from the batch's stream to
     // these streams and joined back (in the captured graph as well)
     static constexpr int kForks = 4;
@@ -55,9 +72,11 @@ struct pflbm_batch {
     int n_work = 0;
     int grid = 0;
     long long nodes = 0;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t graph_exec = nullptr;
-    int graph_n_work = -1;
+    // PFLBM_BATCH_GRAPH_STEPS steps of all members, and of those not resident
+    struct Captured {
+        cudaGraph_t graph = nullptr;
+        cudaGraphExec_t exec = nullptr;
+    } graph, rest_graph;
     void* (*alloc_fn)(size_t, void*) = nullptr;
     void (*free_fn)(void*, size_t, void*) = nullptr;
     void* alloc_ctx = nullptr;
@@ -92,11 +111,12 @@ void bfree(pflbm_batch_t* b, void* p, size_t bytes)
 
 void drop_graph(pflbm_batch_t* b)
 {
-    if (b->graph_exec) cudaGraphExecDestroy(b->graph_exec);
-    if (b->graph) cudaGraphDestroy(b->graph);
-    b->graph_exec = nullptr;
-    b->graph = nullptr;
-    b->graph_n_work = -1;
+    for (pflbm_batch::Captured* g : {&b->graph, &b->rest_graph}) {
+        if (g->exec) cudaGraphExecDestroy(g->exec);
+        if (g->graph) cudaGraphDestroy(g->graph);
+        g->exec = nullptr;
+        g->graph = nullptr;
+    }
 }
 
 // Interleave per-lattice item lists: lattice by lattice (order 0), or the
@@ -156,6 +176,165 @@ std::vector<int4> build_work_staged(const std::vector<pflbm_t*>& hs, const pflbm
     return order_items(per, s.order);
 }
 
+// Groups of the members `idx` with the same size and viscosity mode, largest
+// first, each cut into launches of at most step2_class_capacity().
+std::vector<pflbm_batch::ClassLaunch> build_classes(const pflbm_batch_t* b, std::vector<int> idx,
+                                                    const std::vector<unsigned char>& a0,
+                                                    const std::vector<unsigned char>& a1)
+{
+    std::vector<pflbm_batch::ClassLaunch> out;
+    const int K = step2_class_capacity(b->precision), n = (int)idx.size();
+    auto vv = [&](int i) { return (b->hs[i]->prm.nu_l > 0 && b->hs[i]->prm.nu_g > 0) ? 1 : 0; };
+    std::stable_sort(idx.begin(), idx.end(), [&](int p, int q) {
+        const long long np = (long long)b->hs[p]->nx * b->hs[p]->ny, nq = (long long)b->hs[q]->nx * b->hs[q]->ny;
+        if (np != nq) return np > nq;
+        if (b->hs[p]->nx != b->hs[q]->nx) return b->hs[p]->nx > b->hs[q]->nx;
+        return vv(p) < vv(q);
+    });
+    for (int j = 0; j < n;) {
+        const pflbm_t* h0 = b->hs[idx[j]];
+        int e = j;
+        while (e < n && e - j < K && b->hs[idx[e]]->nx == h0->nx && b->hs[idx[e]]->ny == h0->ny && vv(idx[e]) == vv(idx[j]))
+            ++e;
+        pflbm_batch::ClassLaunch cl;
+        cl.vv = vv(idx[j]);
+        cl.nx = h0->nx;
+        cl.ny = h0->ny;
+        cl.count = e - j;
+        for (int set = 0; set < 2; ++set) {
+            const std::vector<unsigned char>& src = set ? a1 : a0;
+            cl.descs[set].resize(b->args_bytes * cl.count);
+            for (int m = 0; m < cl.count; ++m)
+                std::memcpy(cl.descs[set].data() + b->args_bytes * m, src.data() + b->args_bytes * idx[j + m], b->args_bytes);
+        }
+        out.push_back(std::move(cl));
+        j = e;
+    }
+    return out;
+}
+
+// A device buffer of at least `bytes` (its contents are not kept when it grows).
+int grow(pflbm_batch_t* b, void** p, size_t* cap, size_t bytes)
+{
+    if (bytes <= *cap) return PFLBM_OK;
+    bfree(b, *p, *cap);
+    *p = nullptr;
+    *cap = 0;
+    if (int rc = balloc(b, p, bytes)) return rc;
+    *cap = bytes;
+    return PFLBM_OK;
+}
+
+// FP32 batches of more nodes than this are left to the launches per size group,
+// which then run at 0.9 of the HBM bandwidth: measured, launches -> resident (us
+// per step) 0.20 M nodes 10.5 -> 7.1, 0.39 M 13.8 -> 12.7, 1.7 M 53.0 -> 45.4, 2.5 M
+// 62.2 -> 69.4, 10.4 M 255 -> 276. In 16-bit storage resident is faster at every
+// size: 0.20 M 10.7 -> 5.2, 0.39 M 14.2 -> 9.9, 1.7 M 48.4 -> 34.0, 2.5 M 52.1 ->
+// 48.0, 10.4 M 215 -> 186 (the launches' kernel is bound by latency there).
+constexpr long long kResidentMaxNodes32 = 1LL << 21;
+
+// Waves of members stepped resident, largest members first, each into the first
+// wave with room for its patches; removes them from *idx. Where the patches
+// of the last wave leave SMs idle, the members are cut into more rows of
+// patches, as long as that takes no more waves.
+int plan_waves(pflbm_batch_t* b, std::vector<int>* idx)
+{
+    const int cls = resident_batch_class(b->precision);
+    int coop = 0, sms = 0;
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, b->device);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
+    if (!coop || cls < 0) return PFLBM_OK;
+    if (b->precision == PFLBM_FP32 && b->nodes > kResidentMaxNodes32) return PFLBM_OK;
+    const int n = (int)b->hs.size();
+    struct Member { int i, active; ResidentCut cut; unsigned long long words; };
+    auto pack = [&](double split, std::vector<Member>& ms, std::vector<int>& wave, std::vector<int>& others) {
+        ms.clear();
+        others.clear();
+        for (int i : *idx) {
+            Member m;
+            m.i = i;
+            const pflbm_t* h = b->hs[i];
+            if (cut_resident(h->nx, h->ny, b->precision, h->map, cls, split, &m.cut, &m.active, &m.words) && m.active > 0 &&
+                m.active <= sms)
+                ms.push_back(m);
+            else
+                others.push_back(i);
+        }
+        std::stable_sort(ms.begin(), ms.end(), [](const Member& p, const Member& q) { return p.active > q.active; });
+        std::vector<int> room;
+        wave.assign(ms.size(), 0);
+        for (size_t k = 0; k < ms.size(); ++k) {
+            size_t w = 0;
+            while (w < room.size() && room[w] < ms[k].active) ++w;
+            if (w == room.size()) room.push_back(sms);
+            room[w] -= ms[k].active;
+            wave[k] = (int)w;
+        }
+        return (int)room.size();
+    };
+    std::vector<Member> ms, ms2;
+    std::vector<int> wave, wave2, others, others2;
+    int nw = pack(1.0, ms, wave, others);
+    if (nw == 0) return PFLBM_OK;
+    long long total = 0;
+    for (const Member& m : ms) total += m.active;
+    const double spare = (double)nw * sms / (double)total;
+    for (double split = spare; split > 1.05; split -= 0.1 * (spare - 1.0) + 0.02)
+        if (pack(split, ms2, wave2, others2) <= nw && others2.size() <= others.size()) {
+            ms.swap(ms2);
+            wave.swap(wave2);
+            others.swap(others2);
+            nw = 1 + *std::max_element(wave.begin(), wave.end());
+            break;
+        }
+    std::vector<uint4> items;
+    std::vector<ResidentCut> cuts(n);
+    int most = 0;
+    b->half_words = 0;
+    for (int w = 0; w < nw; ++w) {
+        pflbm_batch::Wave wv{(int)items.size(), 0};
+        unsigned long long at = 0;
+        for (size_t k = 0; k < ms.size(); ++k) {
+            if (wave[k] != w) continue;
+            const Member& m = ms[k];
+            cuts[m.i] = m.cut;
+            for (int p = 0; p < m.cut.px * m.cut.py; ++p)
+                if (m.cut.active[p >> 5] >> (p & 31) & 1u)
+                    items.push_back(make_uint4((unsigned)m.i, (unsigned)p, (unsigned)at, (unsigned)(at >> 32)));
+            at += m.words;
+        }
+        wv.count = (int)items.size() - wv.first;
+        most = std::max(most, wv.count);
+        b->half_words = std::max(b->half_words, at);
+        b->waves.push_back(wv);
+    }
+    b->spill_at = 2 * b->half_words * resident_word_bytes();
+    const size_t bytes = b->spill_at + (size_t)most * resident_spill(b->precision, cls) * 4;
+    const bool fresh = bytes > b->cap_words;
+    void *pi = b->d_items, *pc = b->d_cuts;
+    int rc = grow(b, &pi, &b->cap_items, items.size() * sizeof(uint4));
+    b->d_items = (uint4*)pi;
+    if (!rc) rc = grow(b, &pc, &b->cap_cuts, cuts.size() * sizeof(ResidentCut));
+    b->d_cuts = (ResidentCut*)pc;
+    if (!rc) rc = grow(b, &b->d_words, &b->cap_words, bytes);
+    if (rc) {   // no memory for it: all members take single steps
+        b->waves.clear();
+        return PFLBM_OK;
+    }
+    cudaError_t e = cudaMemcpyAsync(b->d_items, items.data(), items.size() * sizeof(uint4), cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(b->d_cuts, cuts.data(), cuts.size() * sizeof(ResidentCut), cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess && fresh) {
+        e = cudaMemsetAsync(b->d_words, 0, bytes, b->stream);
+        b->res_tag = 0;
+    }
+    // the host vectors go out of scope on return: finish the copies first
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    if (e != cudaSuccess) return set_error(PFLBM_ECUDA, cudaGetErrorString(e));
+    idx->swap(others);
+    return PFLBM_OK;
+}
+
 int upload(pflbm_batch_t* b)
 {
     const int n = (int)b->hs.size();
@@ -177,40 +356,14 @@ int upload(pflbm_batch_t* b)
     // FP32 and 16-bit storage)
     b->by_class = b->precision != PFLBM_FP64 && (b->sched.kernel == 3 || b->sched.kernel == 0);
     b->classes.clear();
+    b->rest.clear();
+    b->waves.clear();
     if (b->by_class) {
-        // groups of lattices with the same size and viscosity mode, largest
-        // first, each cut into launches of at most step2_class_capacity()
-        const int K = step2_class_capacity(b->precision);
         std::vector<int> idx(n);
         for (int i = 0; i < n; ++i) idx[i] = i;
-        auto vv = [&](int i) { return (b->hs[i]->prm.nu_l > 0 && b->hs[i]->prm.nu_g > 0) ? 1 : 0; };
-        std::stable_sort(idx.begin(), idx.end(), [&](int p, int q) {
-            const long long np = (long long)b->hs[p]->nx * b->hs[p]->ny, nq = (long long)b->hs[q]->nx * b->hs[q]->ny;
-            if (np != nq) return np > nq;
-            if (b->hs[p]->nx != b->hs[q]->nx) return b->hs[p]->nx > b->hs[q]->nx;
-            return vv(p) < vv(q);
-        });
-        for (int j = 0; j < n;) {
-            const pflbm_t* h0 = b->hs[idx[j]];
-            int e = j;
-            while (e < n && e - j < K && b->hs[idx[e]]->nx == h0->nx && b->hs[idx[e]]->ny == h0->ny &&
-                   vv(idx[e]) == vv(idx[j]))
-                ++e;
-            pflbm_batch::ClassLaunch cl;
-            cl.vv = vv(idx[j]);
-            cl.nx = h0->nx;
-            cl.ny = h0->ny;
-            cl.count = e - j;
-            for (int set = 0; set < 2; ++set) {
-                const std::vector<unsigned char>& src = set ? a1 : a0;
-                cl.descs[set].resize(b->args_bytes * cl.count);
-                for (int m = 0; m < cl.count; ++m)
-                    std::memcpy(cl.descs[set].data() + b->args_bytes * m, src.data() + b->args_bytes * idx[j + m],
-                                b->args_bytes);
-            }
-            b->classes.push_back(std::move(cl));
-            j = e;
-        }
+        b->classes = build_classes(b, idx, a0, a1);
+        if (int rc = plan_waves(b, &idx)) return rc;
+        if (!b->waves.empty()) b->rest = build_classes(b, idx, a0, a1);
     }
     std::vector<unsigned char> wbytes;
     size_t item = b->staged ? sizeof(int4) : sizeof(int2);
@@ -309,26 +462,26 @@ int check_members(pflbm_t* const* hs, int count, int precision, int device, cuda
 #define PFLBM_BATCH_GRAPH_STEPS 8
 #endif
 
-cudaError_t launch_set(pflbm_batch_t* b, int set);
+cudaError_t launch_set(pflbm_batch_t* b, const std::vector<pflbm_batch::ClassLaunch>& classes, int set);
 
 // nsteps steps from descriptor set `set0` on. With one launch per size group,
 // each group takes its steps back to back on its own forked stream, and the
 // streams join once at the end: a group's lattices need only their own
 // previous step, so small groups run ahead instead of waiting each step for
 // the largest.
-cudaError_t launch_steps(pflbm_batch_t* b, int set0, int nsteps)
+cudaError_t launch_steps(pflbm_batch_t* b, const std::vector<pflbm_batch::ClassLaunch>& classes, int set0, int nsteps)
 {
-    const int nc = (int)b->classes.size();
+    const int nc = (int)classes.size();
     if (!b->by_class || nc <= 1) {
         cudaError_t e = cudaSuccess;
-        for (int s = 0; s < nsteps && e == cudaSuccess; ++s) e = launch_set(b, (set0 + s) & 1);
+        for (int s = 0; s < nsteps && e == cudaSuccess; ++s) e = launch_set(b, classes, (set0 + s) & 1);
         return e;
     }
     const int nf = std::min(nc, (int)pflbm_batch::kForks);
     cudaError_t e = cudaEventRecord(b->fork_ev, b->stream);
     for (int k = 0; k < nf && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(b->fork_stream[k], b->fork_ev, 0);
     for (int c = 0; c < nc && e == cudaSuccess; ++c) {
-        const auto& cl = b->classes[c];
+        const auto& cl = classes[c];
         for (int s = 0; s < nsteps && e == cudaSuccess; ++s)
             e = launch_step2_class(b->precision, cl.vv, cl.descs[(set0 + s) & 1].data(), cl.count, cl.nx, cl.ny,
                                    b->fork_stream[c % nf]);
@@ -338,22 +491,22 @@ cudaError_t launch_steps(pflbm_batch_t* b, int set0, int nsteps)
     return e;
 }
 
-cudaError_t launch_set(pflbm_batch_t* b, int set)
+cudaError_t launch_set(pflbm_batch_t* b, const std::vector<pflbm_batch::ClassLaunch>& classes, int set)
 {
     if (b->staged)
         return launch_step_staged_batch(b->precision, b->d_args[set], (const int4*)b->d_work, b->n_work, b->grid,
                                         b->stream);
     if (b->by_class) {
-        const int nc = (int)b->classes.size();
+        const int nc = (int)classes.size();
         if (nc == 1)
-            return launch_step2_class(b->precision, b->classes[0].vv, b->classes[0].descs[set].data(),
-                                      b->classes[0].count, b->classes[0].nx, b->classes[0].ny, b->stream);
+            return launch_step2_class(b->precision, classes[0].vv, classes[0].descs[set].data(), classes[0].count,
+                                      classes[0].nx, classes[0].ny, b->stream);
         const int nf = std::min(nc, (int)pflbm_batch::kForks);   // streams made by upload()
         cudaError_t e = cudaEventRecord(b->fork_ev, b->stream);
         for (int k = 0; k < nf && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(b->fork_stream[k], b->fork_ev, 0);
         // largest groups first, dealt round-robin over the forked streams
         for (int c = 0; c < nc && e == cudaSuccess; ++c) {
-            const auto& cl = b->classes[c];
+            const auto& cl = classes[c];
             e = launch_step2_class(b->precision, cl.vv, cl.descs[set].data(), cl.count, cl.nx, cl.ny,
                                    b->fork_stream[c % nf]);
         }
@@ -365,24 +518,92 @@ cudaError_t launch_set(pflbm_batch_t* b, int set)
                              std::max(1, b->sched.tiles_per_item), b->grid, b->stream);
 }
 
-int ensure_graph(pflbm_batch_t* b)
+int ensure_graph(pflbm_batch_t* b, const std::vector<pflbm_batch::ClassLaunch>& classes, pflbm_batch::Captured* g)
 {
-    if (b->graph_exec && b->graph_n_work == b->n_work) return PFLBM_OK;
-    drop_graph(b);
+    if (g->exec) return PFLBM_OK;
     cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return set_error(PFLBM_ECUDA, cudaGetErrorString(e));
-    cudaError_t e1 = launch_steps(b, 0, PFLBM_BATCH_GRAPH_STEPS);
-    e = cudaStreamEndCapture(b->stream, &b->graph);
+    cudaError_t e1 = launch_steps(b, classes, 0, PFLBM_BATCH_GRAPH_STEPS);
+    e = cudaStreamEndCapture(b->stream, &g->graph);
     if (e1 != cudaSuccess || e != cudaSuccess) {
         drop_graph(b);
         return set_error(PFLBM_ECUDA, "batch: graph capture failed");
     }
-    e = cudaGraphInstantiate(&b->graph_exec, b->graph, 0);
+    e = cudaGraphInstantiate(&g->exec, g->graph, 0);
     if (e != cudaSuccess) {
         drop_graph(b);
         return set_error(PFLBM_ECUDA, cudaGetErrorString(e));
     }
-    b->graph_n_work = b->n_work;
+    return PFLBM_OK;
+}
+
+// n steps of the members in `classes` (all members where the kernel has no
+// size groups) from parity `phase` on, by graph replays where asked.
+int step_launches(pflbm_batch_t* b, const std::vector<pflbm_batch::ClassLaunch>& classes, pflbm_batch::Captured* g, int phase,
+                  int64_t n)
+{
+    static_assert(PFLBM_BATCH_GRAPH_STEPS >= 2 && PFLBM_BATCH_GRAPH_STEPS % 2 == 0, "an even step count per graph");
+    auto single = [&]() -> int {
+        cudaError_t e = launch_set(b, classes, phase);
+        if (e != cudaSuccess) return set_error(PFLBM_ECUDA, cudaGetErrorString(e));
+        phase ^= 1;
+        --n;
+        return PFLBM_OK;
+    };
+    if (phase == 1 && n > 0)
+        if (int rc = single()) return rc;
+    if (b->sched.use_graph && n >= PFLBM_BATCH_GRAPH_STEPS) {
+        if (int rc = ensure_graph(b, classes, g)) return rc;
+        for (; n >= PFLBM_BATCH_GRAPH_STEPS; n -= PFLBM_BATCH_GRAPH_STEPS) {
+            cudaError_t e = cudaGraphLaunch(g->exec, b->stream);
+            if (e != cudaSuccess) return set_error(PFLBM_ECUDA, cudaGetErrorString(e));
+        }
+    }
+    while (n > 0)
+        if (int rc = single()) return rc;
+    return PFLBM_OK;
+}
+
+// Runs of at least this many steps take the resident path (a wave costs about
+// 20 us more than its steps), in launches of at most kResidentMaxSteps (even).
+constexpr int64_t kResidentMinSteps = 16;
+constexpr int kResidentMaxSteps = 1024;
+
+bool capturing(cudaStream_t stream)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
+}
+
+int step_waves(pflbm_batch_t* b, int64_t n)
+{
+    const int cls = resident_batch_class(b->precision);
+    for (const pflbm_batch::Wave& w : b->waves) {
+        int phase = b->phase;
+        for (int64_t left = n; left > 0;) {
+            const int c = (int)std::min<int64_t>(left, kResidentMaxSteps);
+            cudaError_t e = cudaSuccess;
+            if (b->res_tag > UINT_MAX - 2u * kResidentMaxSteps) {   // tags start again
+                e = cudaMemsetAsync(b->d_words, 0, b->spill_at, b->stream);
+                b->res_tag = 0;
+            }
+            ResidentWave a{};
+            a.args = b->d_args[phase];
+            a.cuts = b->d_cuts;
+            a.items = b->d_items + w.first;
+            a.words = b->d_words;
+            a.half = b->half_words;
+            a.spill = (uint32_t*)((char*)b->d_words + b->spill_at);
+            a.tag = b->res_tag;
+            a.steps = c;
+            a.n_items = w.count;
+            if (e == cudaSuccess) e = launch_resident_wave(b->precision, a, cls, b->stream);
+            if (e != cudaSuccess) return set_error(PFLBM_ECUDA, cudaGetErrorString(e));
+            b->res_tag += (unsigned)c;
+            phase ^= c & 1;
+            left -= c;
+        }
+    }
     return PFLBM_OK;
 }
 
@@ -449,7 +670,7 @@ int pflbm_batch_step(pflbm_batch_t* b, int64_t n)
     for (size_t i = 0; i < b->hs.size(); ++i) {
         pflbm_t* h = b->hs[i];
         if (h->hstatus && (h->hstatus[0] & 4))
-            return set_error(PFLBM_ETIMEOUT, "batch: a wait for staged data in the step kernel gave up");
+            return set_error(PFLBM_ETIMEOUT, "batch: a wait in the step kernel gave up");
         if (h->hstatus && h->hstatus[0] != 0)
             return set_error(PFLBM_ENUMERIC, "batch: NaN or |u| >= 0.3 detected on the device");
         if (h->init_pending) {
@@ -460,27 +681,14 @@ int pflbm_batch_step(pflbm_batch_t* b, int64_t n)
     if (stale) {  // a member was stepped on its own: rewrite the descriptors
         if (int rc = upload(b)) return rc;
     }
-    int64_t left = n;
-    if (b->phase == 1) {
-        cudaError_t e = launch_set(b, 1);
-        if (e != cudaSuccess) return set_error(PFLBM_ECUDA, cudaGetErrorString(e));
-        b->phase = 0;
-        --left;
+    if (!b->waves.empty() && n >= kResidentMinSteps && !capturing(b->stream)) {
+        if (int rc = step_waves(b, n)) return rc;
+        if (!b->rest.empty())
+            if (int rc = step_launches(b, b->rest, &b->rest_graph, b->phase, n)) return rc;
+    } else if (int rc = step_launches(b, b->classes, &b->graph, b->phase, n)) {
+        return rc;
     }
-    static_assert(PFLBM_BATCH_GRAPH_STEPS >= 2 && PFLBM_BATCH_GRAPH_STEPS % 2 == 0, "an even step count per graph");
-    if (b->sched.use_graph && left >= PFLBM_BATCH_GRAPH_STEPS) {
-        if (int rc = ensure_graph(b)) return rc;
-        for (; left >= PFLBM_BATCH_GRAPH_STEPS; left -= PFLBM_BATCH_GRAPH_STEPS) {
-            cudaError_t e = cudaGraphLaunch(b->graph_exec, b->stream);
-            if (e != cudaSuccess) return set_error(PFLBM_ECUDA, cudaGetErrorString(e));
-        }
-    }
-    while (left > 0) {
-        cudaError_t e = launch_set(b, b->phase);
-        if (e != cudaSuccess) return set_error(PFLBM_ECUDA, cudaGetErrorString(e));
-        b->phase ^= 1;
-        --left;
-    }
+    b->phase ^= (int)(n & 1);
     for (pflbm_t* h : b->hs) {
         if (n & 1) h->cur ^= 1;
         h->steps += n;
@@ -522,6 +730,9 @@ void pflbm_batch_destroy(pflbm_batch_t* b)
     if (b->fork_ev) cudaEventDestroy(b->fork_ev);
     for (int k = 0; k < 2; ++k) bfree(b, b->d_args[k], b->args_bytes * b->cap_lattices);
     bfree(b, b->d_work, sizeof(int4) * b->cap_work);
+    bfree(b, b->d_items, b->cap_items);
+    bfree(b, b->d_cuts, b->cap_cuts);
+    bfree(b, b->d_words, b->cap_words);
     delete b;
 }
 

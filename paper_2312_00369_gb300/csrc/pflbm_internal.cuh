@@ -246,6 +246,11 @@ bool plan_resident(int nx, int ny, int precision, const SolidMap& map, int max_c
                    ResidentPlan* out);
 size_t resident_word_bytes();
 int resident_batch_class(int precision);              // patch class of batches; < 0: none
+// The cut of a batch's member: the fewest patches of the class (split = 1), or
+// `split` times as many rows of them. Gives its active patches and its exchange
+// words (one buffer).
+bool cut_resident(int nx, int ny, int precision, const SolidMap& map, int cls, double split, ResidentCut* cut,
+                  int* n_active, unsigned long long* half_words);
 int resident_spill(int precision, int cls);           // 32-bit words of list overflow per CTA
 cudaError_t launch_resident_wave(int precision, const ResidentWave& w, int cls, cudaStream_t stream);
 cudaError_t launch_resident(pflbm_t* h, const ResidentPlan& plan, int steps);

@@ -130,6 +130,11 @@ __device__ __forceinline__ int slot_of(const Rect& r, int lx, int ly)
     return 6 * r.w + ly * 6 + 3 + lx - (r.w - 3);
 }
 
+// Words of a patch in one buffer: its types' slots, then the heartbeat in a line
+// of its own.
+constexpr int kHeartbeat = 8;
+__host__ __device__ __forceinline__ int patch_words(const ResidentCut& c) { return (kTypes * c.max_slots + 7) / 8 * 8 + kHeartbeat; }
+
 // Shared memory of a patch of at most WM x HM nodes: byte offsets of the
 // arrays. Row and plane strides are constants, so a pull's offset is an
 // immediate of its load.
@@ -499,25 +504,6 @@ __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ R
         if (!own && want) sRing[atomicAdd(&s_n[2], 1)] = (uint16_t)c;
     }
     __syncthreads();
-    // heartbeats: one word of every patch that this one's halo reaches, so that
-    // neither runs ahead of the other even where only one of them wants values
-    for (int c = tid; c < area; c += NT) {
-        const int ly = c / rs - kHaloY, lx = c % rs - kHaloX, gy = r.y0 + ly;
-        if (lx < -3 || lx > r.w + 2 || gy < 1 || gy > ny - 2) continue;
-        const int gx = wrapn(r.x0 + lx, nx);
-        const int of = ((gy * cut.py - 1) / cut.rows) * cut.px + ((gx / N + 1) * cut.px - 1) / cut.units;
-        if (of == id || !(cut.active[of >> 5] >> (of & 31) & 1u)) continue;
-        if (atomicOr(&s_seen[of >> 5], 1u << (of & 31)) >> (of & 31) & 1u) continue;
-        const int at = atomicAdd(&s_n[0], 1);
-        const uint32_t u = (uint32_t)(cut.px * cut.py * kTypes * cut.max_slots + of);
-        if (at < L::CAP) {
-            sPoll[at] = u;
-            sPollC[at] = (uint16_t)(cells - 1);
-        } else if (at < L::MAXLIST) {
-            gPoll[at] = u;
-            gPollC[at] = (uint32_t)(cells - 1);
-        }
-    }
     for (int p = 0; p < kTypes; ++p) {
         for (int c0 = tid & ~31; c0 < area; c0 += NT) {
             const int c = c0 + (tid & 31), ly = c / rs - kHaloY, lx = c % rs - kHaloX;
@@ -540,8 +526,9 @@ __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ R
                     const int i = ((gx / N + 1) * cut.px - 1) / cut.units, j = (gy * cut.py - 1) / cut.rows;
                     const int from = j * cut.px + i;
                     const Rect o = patch_rect<N>(cut, from, nx);
-                    const uint32_t u = (uint32_t)p << 28 | (uint32_t)((from * kTypes + p) * cut.max_slots +
+                    const uint32_t u = (uint32_t)p << 28 | (uint32_t)(from * patch_words(cut) + p * cut.max_slots +
                                                                       slot_of(o, gx - o.x0, gy - o.y0));
+                    atomicOr(&s_seen[from >> 5], 1u << (from & 31));
                     if (at < L::CAP) {
                         sPoll[at] = u;
                         sPollC[at] = (uint16_t)c;
@@ -551,6 +538,27 @@ __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ R
                     }
                 }
             }
+        }
+    }
+    __syncthreads();
+    // heartbeats: one word of every patch that this one's halo reaches and that
+    // it wants nothing else from, so that neither runs ahead of the other
+    for (int c = tid; c < area; c += NT) {
+        const int ly = c / rs - kHaloY, lx = c % rs - kHaloX, gy = r.y0 + ly;
+        if (lx < -3 || lx > r.w + 2 || gy < 1 || gy > ny - 2) continue;
+        const int gx = wrapn(r.x0 + lx, nx);
+        const int of = ((gy * cut.py - 1) / cut.rows) * cut.px + ((gx / N + 1) * cut.px - 1) / cut.units;
+        if (of == id || !(cut.active[of >> 5] >> (of & 31) & 1u)) continue;
+        if (s_seen[of >> 5] >> (of & 31) & 1u) continue;
+        if (atomicOr(&s_seen[of >> 5], 1u << (of & 31)) >> (of & 31) & 1u) continue;
+        const int at = atomicAdd(&s_n[0], 1);
+        const uint32_t u = (uint32_t)((of + 1) * patch_words(cut) - kHeartbeat);
+        if (at < L::CAP) {
+            sPoll[at] = u;
+            sPollC[at] = (uint16_t)(cells - 1);
+        } else if (at < L::MAXLIST) {
+            gPoll[at] = u;
+            gPollC[at] = (uint32_t)(cells - 1);
         }
     }
     __syncthreads();
@@ -706,9 +714,8 @@ __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ R
         constexpr int NS = (L::kPhi - L::kS) / (int)sizeof(S), NW = (L::kPhi - L::kS) / 4;   // elements of sS and sG0
         Word* buf = ll + (s & 1) * q.ll_half;
         {
-            Word* to = buf + (unsigned long long)id * kTypes * cut.max_slots * WPT;
-            if (tid < WPT)
-                st_word(buf + (unsigned long long)(cut.px * cut.py * kTypes * cut.max_slots + id) * WPT + tid, 0u, 0u, 0u, tag);
+            Word* to = buf + (unsigned long long)id * patch_words(cut) * WPT;
+            if (tid < WPT) st_word(to + (patch_words(cut) - kHeartbeat) * WPT + tid, 0u, 0u, 0u, tag);
             for (int e = tid; e < n_pub; e += NT) {
                 const uint32_t u = e < L::CAP ? sPub[e] : gPub[e];
                 const int c = (int)(u & 0x1fffu);
@@ -973,7 +980,7 @@ bool plan_resident(int nx, int ny, int precision, const SolidMap& map, int max_c
                 if (h > c.hm || lanes > c.p * c.nt) break;
                 const double cost = ((precision == PFLBM_FP64 ? 100.0 : 2.4) * ((lanes + 31) / 32 * 32 * unit) +
                                      4.3 * 2 * (w2 + h)) *
-                                    (lw == 16 || lw == 32 ? 0.9 : 1.0);
+                                    (lw == 16 ? 0.88 : lw == 32 ? 0.94 : 1.0);
                 if (cost >= best) break;      // fewer rows of patches only cost more
                 ResidentCut cut{};
                 cut.px = px;
@@ -999,7 +1006,7 @@ bool plan_resident(int nx, int ny, int precision, const SolidMap& map, int max_c
                 const int per = ((lanes + c.p - 1) / c.p + 31) / 32 * 32;
                 // the exchange and the ring want threads too
                 out->nt = per < 256 ? 256 : per;
-                out->words = 2ull * px * py * (kTypes * cut.max_slots + 1) * (precision == PFLBM_FP64 ? 2 : 1);
+                out->words = 2ull * px * py * patch_words(cut) * (precision == PFLBM_FP64 ? 2 : 1);
                 out->bytes = out->words * sizeof(Word) + (size_t)n * spill_of(precision, k) * 4;
                 break;
             }
@@ -1010,6 +1017,31 @@ bool plan_resident(int nx, int ny, int precision, const SolidMap& map, int max_c
 
 size_t resident_word_bytes() { return sizeof(Word); }
 int resident_batch_class(int precision) { return precision == PFLBM_FP64 ? -1 : 2; }
+bool cut_resident(int nx, int ny, int precision, const SolidMap& map, int cls, double split, ResidentCut* cut, int* n_active,
+                  unsigned long long* half_words)
+{
+    if (map.sum.empty() || precision == PFLBM_FP64) return false;
+    const Class c = class_of(precision, cls);
+    const int units = (nx + 1) / 2, rows = ny - 2;
+    *cut = ResidentCut{};
+    cut->px = (units + c.wm / 2 - 1) / (c.wm / 2);
+    const int least = (rows + c.hm - 1) / c.hm, most = rows / 8 > least ? rows / 8 : least;
+    cut->py = (int)(least * split) < most ? (int)(least * split) : most;
+    if (cut->py < least) cut->py = least;
+    if ((long long)cut->px * cut->py > kMaxPatches) return false;
+    cut->units = units;
+    cut->rows = rows;
+    cut->max_slots = 6 * ((units + cut->px - 1) / cut->px * 2 + (rows + cut->py - 1) / cut->py);
+    int n = 0;
+    for (int i = 0; i < cut->px * cut->py; ++i)
+        if (patch_active(map, patch_rect<2>(*cut, i, nx), nx)) {
+            cut->active[i >> 5] |= 1u << (i & 31);
+            ++n;
+        }
+    *n_active = n;
+    *half_words = (unsigned long long)cut->px * cut->py * patch_words(*cut);
+    return true;
+}
 int resident_spill(int precision, int cls) { return spill_of(precision, cls); }
 
 cudaError_t launch_resident(pflbm_t* h, const ResidentPlan& pl, int steps)

@@ -159,3 +159,42 @@ def test_no_index_outside_its_buffer():
                        timeout=600)
     assert r.returncode == 0, r.stderr[-2000:]
     assert r.stdout.strip().endswith("violations 0"), r.stdout
+
+
+BATCH = [  # mask, nx, ny, options: 1 to 100 patches, odd widths, one lattice that does not fit
+    (_frame, 64, 32, {}), (_slope, 128, 64, {}), (_blocks, 65, 33, dict(chi_case=1)),
+    (_disc, 256, 128, dict(nu_l=0.3, nu_g=0.05, gx=2e-6, gy=-1e-6)), (_frame, 3, 9, {}), (_slope, 512, 256, {}),
+    (_frame, 301, 203, {}), (_frame, 1200, 400, {}), (_disc, 512, 256, dict(dgdt_mode=1)),
+]
+
+
+@pytest.mark.parametrize("precision", ["fp32", "bf16", "fp16"])
+def test_resident_batch_equals_single_steps(precision):
+    from paper_2312_00369_gb300.pflbm import Batch
+    stream = torch.cuda.Stream()
+    many = [_solver(*c[:3], precision, "default", dict(c[3], stream=stream)) for c in BATCH]
+    one = [_solver(*c[:3], precision, "global", dict(c[3], stream=stream)) for c in BATCH]
+    b = Batch(many)
+    # resident runs of either parity, single steps between, a member stepped
+    # alone, a change of members
+    for n in (16, 3, 37):
+        b.step(n)
+        for s in one:
+            s.step(n)
+    many[1].step(5)
+    one[1].step(5)
+    b.step(20)
+    for s in one:
+        s.step(20)
+    b.set(many[:4])
+    b.step(17)
+    for s in one[:4]:
+        s.step(17)
+    for c, x, y in zip(BATCH, many, one):
+        assert x.steps == y.steps
+        for p, q, what in zip(_state(x), _state(y), ("phi", "u", "p", "mass")):
+            assert np.array_equal(p, q), (c[1:3], what)
+        x.check()
+    b.close()
+    for s in many + one:
+        s.close()
