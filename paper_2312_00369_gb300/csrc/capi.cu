@@ -142,7 +142,6 @@ void release(pflbm_t* h)
     dfree(h, h->pop[1], s.pop);
     dfree(h, h->sprev, s.sprev);
     dfree(h, h->phi0, s.N * sizeof(double));
-    dfree(h, h->mu0, s.N * sizeof(double));
     dfree(h, h->red, s.red);
     dfree(h, h->pts, s.pts);
     dfree(h, h->out, h->out_bytes);
@@ -184,8 +183,7 @@ int post_status_copy(pflbm_t* h)
 int materialize(pflbm_t* h)
 {
     if (!h->init_pending) return PFLBM_OK;
-    CK(launch_init_populations(h));
-    CK(cudaMemsetAsync(h->dstatus, 0, sizeof(int), h->stream));
+    CK(launch_init_populations(h));   // clears the device status word too
     if (h->hstatus) h->hstatus[0] = 0;
     h->init_pending = false;
     return PFLBM_OK;
@@ -357,6 +355,8 @@ size_t pflbm_footprint_bytes(int nx, int ny, int precision)
 {
     if (nx < 1 || ny < 1) return 0;
     Sizes s = sizes_of(nx, ny, precision);
+    // (of the 26 bytes per node beside the state, 8 are an allowance for the
+    // exchange memory of resident runs, allocated on first use)
     return 2 * s.pop + s.sprev + s.wet + s.N * (1 + 1 + 8 + 8 + 8) + s.red + s.pts + s.tiles + 16 +
            (size_t)nx * ny * 4 * sizeof(double) +
            (precision != PFLBM_FP64 ? tma_sets_bytes() + staged_flags_bytes(nx, ny) + node_words_bytes(nx, ny) +
@@ -439,7 +439,6 @@ int pflbm_create_ex(pflbm_t** out, const pflbm_params_t* prm)
     ALLOC(pop[1], s.pop);
     ALLOC(sprev, s.sprev);
     ALLOC(phi0, s.N * sizeof(double));
-    ALLOC(mu0, s.N * sizeof(double));
     ALLOC(red, s.red);
     ALLOC(pts, s.pts);
     ALLOC(dstatus, sizeof(int) * 4);
@@ -599,6 +598,7 @@ int pflbm_init_phi(pflbm_t* h, const double* phi)
     CK(cudaMemcpy2DAsync(h->phi0, h->pitch * sizeof(double), phi, h->nx * sizeof(double), h->nx * sizeof(double),
                          h->ny, cudaMemcpyHostToDevice, h->stream));
     h->replace_phi = false;
+    h->phi0_nonneg = false;
     h->init_pending = true;
     CK(cudaStreamSynchronize(h->stream));   // phi is a caller buffer: done with it on return
     h->steps = 0;

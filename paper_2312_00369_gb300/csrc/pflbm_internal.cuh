@@ -113,6 +113,16 @@ cudaError_t launch_contact_angle3d(const uint8_t* cls, const double* d_phi, int 
                                    const Wall3& w, double* pts, int cap, int* d_count, double* d_out,
                                    cudaStream_t stream);
 
+// Distance from its centre beyond which a droplet's profile 1/2 + 1/2 tanh(2 (R -
+// r) / W) is exactly 0. FP64: |R| + 10 W (tanh(-20) rounds to -1). FP32:
+// |R| + 6 W, since tanhf is exactly -1 at an argument of -12 and beyond (checked
+// for every float from -9.02 to -24); but a field that may hold negative values keeps
+// 10 W, within which they have always been raised to 0.
+inline double droplet_reach(bool fp64, bool nonneg, double R, double W)
+{
+    return (R < 0 ? -R : R) + (fp64 || !nonneg ? 10.0 : 6.0) * W;
+}
+
 struct Params {           // derived parameters (Sec. 2.1-2.2), in FP64
     double beta, kappa, alpha, tau_f, tau_g, rho_l, rho_g, W, sigma, M;
     double nu_l, nu_g;    // both > 0: variable viscosity
@@ -183,8 +193,7 @@ struct pflbm {
     double* av = nullptr;         // a_v [N]
     void* pop[2] = {nullptr, nullptr};  // f then g, each [9][ny][pitch], ping-pong
     void* sprev = nullptr;        // u.grad(phi) history [N]
-    double* phi0 = nullptr;       // initial-field staging / ghost-filled phi [N]
-    double* mu0 = nullptr;        // initial chemical potential [N]
+    double* phi0 = nullptr;       // initial-field staging [N]
     double* red = nullptr;        // reduction scratch
     double* pts = nullptr;        // contact-angle points (2 * pts_cap)
     int pts_cap = 0;
@@ -195,6 +204,7 @@ struct pflbm {
     int* hstatus = nullptr;       // pinned host mirror
     int cur = 0;                  // which pop buffer holds the current state
     bool replace_phi = true;
+    bool phi0_nonneg = true;      // phi0 holds droplets only
     bool init_pending = false;    // phi0 set, populations not yet built
     int64_t steps = 0;
     size_t bytes_allocated = 0;

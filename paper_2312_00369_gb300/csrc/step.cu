@@ -362,10 +362,12 @@ StepArgs<PREC> make_args(pflbm_t* h)
 // [ylo, yhi), combined with the field by maximum (a replacing call cleared it).
 // F32: the profile in FP32 (solves whose arithmetic is FP32 or 16-bit storage;
 // the FP64 tanh is slow on this part), else in FP64.
-template <bool F32>
+// REPLACE: the box is the whole lattice and the field is written everywhere (a
+// replacing call on a small lattice: one launch instead of a clear and a launch).
+template <bool F32, bool REPLACE>
 __global__ void k_init_droplet(const uint8_t* __restrict__ cls, double* __restrict__ phi, int nx, int ny,
                                int pitch, int xlo, int xw, int ylo, int yhi, double x0, double y0, double R,
-                               double W)
+                               double W, double reach)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     int y = ylo + blockIdx.y * blockDim.y + threadIdx.y;
@@ -373,129 +375,191 @@ __global__ void k_init_droplet(const uint8_t* __restrict__ cls, double* __restri
     int x = (xlo + i) % nx;
     if (x < 0) x += nx;
     size_t k = (size_t)y * pitch + x;
+    if (REPLACE) phi[k] = 0.0;
     if (!zeta_of(cls[k])) return;
     double dx = fabs((double)x - x0);
     if (dx >= nx) dx = fmod(dx, (double)nx);   // exact; only for a period or more
     if (dx > 0.5 * nx) dx = nx - dx;           // x-periodic distance
     const double dy = (double)y - y0, r2 = dx * dx + dy * dy;
-    // beyond |R| + 10 W the profile is 0 in FP64 (tanh(-20) rounds to -1):
-    // the bounding box's corners are skipped like the nodes outside it
-    const double reach = fabs(R) + 10.0 * W;
+    // beyond `reach` the profile is 0 (droplet_reach): the bounding box's
+    // corners are skipped like the nodes outside it
     if (r2 > reach * reach) return;
     const double v = F32 ? (double)(0.5f + 0.5f * tanhf(2.0f * ((float)R - sqrtf((float)r2)) / (float)W))
                          : 0.5 + 0.5 * tanh(2.0 * (R - sqrt(r2)) / W);
-    if (v > phi[k]) phi[k] = v;
+    if (REPLACE || v > phi[k]) phi[k] = v;
 }
 
-template <typename C>
-__global__ void k_ghost_fill(const uint8_t* __restrict__ cls, const C* __restrict__ wet, double* __restrict__ phi,
-                             int nx, int ny, int pitch)
+// The initial state in one pass: ghost values of phi0 (Sec. 2.2.2), mu of the
+// initial field (Eq. chemical_potencial2), the u.grad(phi) history of the first
+// step, and the post-collision arrays that the first pull turns into f = 0,
+// g = g^eq(phi0, mu). A CTA takes a 32 x 8 tile: phi0 and the classes within
+// three nodes, ghost values within two, mu within one.
+//
+// mu and the history are evaluated in the precision of the step's arithmetic
+// (C): FP64 for FP64 solves, FP32 otherwise (a 32-bit state stores mu only
+// through g_i^eq = w_i alpha mu, rounded to 32 or 16 bits; phi = sum g_i stays
+// exact through g_0). The products with alpha, the rounding residuals and g_0
+// are FP64.
+//
+// Bound by the writes (80 B per node in FP32, 44 in 16-bit storage) where the
+// tile holds no phase; FP64 instructions (19 cycles a warp and SM) are what the
+// rest costs, so they are spent once per source node instead of once per
+// direction, and not at all where phi0 is 0 within three nodes of the tile
+// (both halves of g^eq vanish; most tiles of a lattice of droplets). Measured, 4096
+// x 2048 with 64 droplets, three passes (ghosts, mu, populations) -> this one:
+// BF16 1087 -> 153 us, FP32 672 -> 173 us.
+template <int PREC>
+__global__ void __launch_bounds__(TX * TY) k_init_state(const uint8_t* __restrict__ cls,
+                                                        const typename Store<PREC>::C* __restrict__ wet,
+                                                        const double* __restrict__ phi0, Planes<PREC> P,
+                                                        typename Store<PREC>::C* __restrict__ sprev, int* status, int nx,
+                                                        int ny, int pitch, size_t plane, Params q)
 {
-    int x = blockIdx.x * blockDim.x + threadIdx.x;
-    int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= nx || y >= ny) return;
-    size_t k = (size_t)y * pitch + x;
-    const uint8_t code = cls[k];
-    uint8_t c = code & CLS_MASK;
-    if (c == CLS_INTERIOR) { phi[k] = 0.0; return; }
-    if (c != CLS_GHOST) return;
-    if (code & (F_GHOST_UP | F_GHOST_DOWN)) {
-        // the mirror node is zeta = 1, never a ghost: no ordering hazard
-        phi[k] = robin_ghost<double>(phi[(code & F_GHOST_UP) ? k + pitch : k - pitch], (double)wet[k]);
+    using T = Store<PREC>;
+    using C = typename T::C;
+    using S = typename T::S;
+    constexpr int W3 = TX + 6, H3 = TY + 6, W1 = TX + 2, H1 = TY + 2;
+    constexpr int kG = T::kNorm ? 0 : 1;   // 16-bit: the unused plane of g is cleared too; else it is that of g_0
+    __shared__ double s_phi[H3][W3];
+    __shared__ uint8_t s_cls[H3][W3];
+    __shared__ C s_mu[H1][W1];
+    __shared__ C s_g[2][H1][W1];                             // w alpha mu of the axes and the diagonals
+    __shared__ double s_res[T::kAbsorb ? 2 : 1][H1][W1];     // and what storage rounds off them
+    const int tid = threadIdx.y * TX + threadIdx.x;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *status = 0;
+
+    bool phase = false;
+    for (int p = tid; p < H3 * W3; p += TX * TY) {
+        const int py = p / W3, px = p - py * W3, y = y0 - 3 + py;
+        uint8_t c = CLS_OUT;
+        double v = 0.0;
+        if (y >= 0 && y < ny) {
+            const size_t k = (size_t)y * pitch + wrapn(x0 - 3 + px, nx);
+            c = cls[k];
+            if (zeta_of(c)) v = phi0[k];
+        }
+        s_cls[py][px] = c;
+        s_phi[py][px] = v;
+        phase = phase || __double_as_longlong(v) != 0;
+    }
+    phase = __syncthreads_or(phase);
+
+    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
+    const bool mine = x < nx && y < ny;
+    const size_t k = (size_t)y * pitch + x;
+    const S zero = T::template st<0>(C(0));
+    if (mine) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) P.f[i * plane + k] = zero;
+    }
+    const uint8_t code = s_cls[threadIdx.y + 3][threadIdx.x + 3];
+    if (!phase) {
+        if (mine) {
+#pragma unroll
+            for (int i = kG; i < 9; ++i) P.g[i * plane + k] = zero;
+            P.g0[k] = T::g0_from_double(0.0);
+            sprev[k] = C(0);
+        }
         return;
     }
-    double num = 0.0, den = 0.0;
+
+    // ghost values within two nodes of the tile
+    for (int p = tid; p < (TY + 4) * (TX + 4); p += TX * TY) {
+        const int py = p / (TX + 4) + 1, px = p % (TX + 4) + 1;
+        const uint8_t c = s_cls[py][px];
+        if (c == CLS_OUT || (c & CLS_MASK) != CLS_GHOST) continue;
+        if (c & (F_GHOST_UP | F_GHOST_DOWN)) {
+            const size_t m = (size_t)(y0 - 3 + py) * pitch + wrapn(x0 - 3 + px, nx);
+            s_phi[py][px] = robin_ghost<double>(s_phi[(c & F_GHOST_UP) ? py + 1 : py - 1][px], (double)wet[m]);
+            continue;
+        }
+        double num = 0.0, den = 0.0;
+        for (int j = 1; j < 9; ++j)
+            if (zeta_of(s_cls[py + cy(j)][px + cx(j)])) { num += s_phi[py + cy(j)][px + cx(j)]; den += 1.0; }
+        s_phi[py][px] = num / den;
+    }
+    __syncthreads();
+
+    // mu within one node, and what its neighbours store of it
+    const double ka = 1.0 / 9.0 * q.alpha, kd = 1.0 / 36.0 * q.alpha;
+    for (int p = tid; p < H1 * W1; p += TX * TY) {
+        const int r = p / W1, c1 = p - r * W1, py = r + 2, px = c1 + 2;
+        const uint8_t cd = s_cls[py][px];
+        C m = C(0), ga = C(0), gd = C(0);
+        double ra = 0.0, rd = 0.0;
+        if (zeta_of(cd)) {
+            auto at = [&](int dx, int dy) { return (C)s_phi[py + dy][px + dx]; };
+            const C c = at(0, 0);
+            const C E = at(1, 0), Wv = at(-1, 0), N = at(0, 1), So = at(0, -1);
+            const C NE = at(1, 1), NW = at(-1, 1), SW = at(-1, -1), SE = at(1, -1);
+            // multiplications by rounded reciprocals: division is slow
+            const C lap = ((E + Wv) + (N + So)) * (C(2) / C(3)) + ((NE + NW) + (SE + SW)) * (C(1) / C(6)) - c * (C(10) / C(3));
+            const size_t kk = (size_t)(y0 - 3 + py) * pitch + wrapn(x0 - 3 + px, nx);
+            const C wv = (cd & F_WET) ? wet[kk] : C(0);
+            m = C(4) * (C)q.beta * c * (c - C(1)) * (c - C(0.5)) - (C)q.kappa * lap - wv * (c - c * c);
+            if (px >= 3 && px < TX + 3 && py >= 3 && py < TY + 3 && x0 + px - 3 < nx) {
+                // u at t = 0 from f = 0: u = F / (2 rho), F = mu grad(phi) + rho g; the
+                // history of the first step is u.grad(phi)
+                const C gpx = (E - Wv) * (C(1) / C(3)) + ((NE + SE) - (NW + SW)) * (C(1) / C(12));
+                const C gpy = (N - So) * (C(1) / C(3)) + ((NE + NW) - (SE + SW)) * (C(1) / C(12));
+                const C rho = (C)q.rho_g + (C)(q.rho_l - q.rho_g) * c;
+                const C half_inv_rho = C(0.5) / rho;
+                const C ux = (m * gpx + rho * (C)q.gx) * half_inv_rho, uy = (m * gpy + rho * (C)q.gy) * half_inv_rho;
+                sprev[kk] = ux * gpx + uy * gpy;
+            }
+            ga = gd = m;                   // 0 keeps its sign
+            if (m != C(0)) {
+                const double va = ka * (double)m, vd = kd * (double)m;
+                ga = (C)va;
+                gd = (C)vd;
+                if (T::kAbsorb) {
+                    ra = va - (double)T::template ld<1>(T::template st<1>(ga));
+                    rd = vd - (double)T::template ld<5>(T::template st<5>(gd));
+                }
+            }
+        }
+        s_mu[r][c1] = m;
+        s_g[0][r][c1] = ga;
+        s_g[1][r][c1] = gd;
+        if constexpr (T::kAbsorb) {
+            s_res[0][r][c1] = ra;
+            s_res[1][r][c1] = rd;
+        }
+    }
+    __syncthreads();
+
+    if (!mine) return;
+    if (kG == 0) P.g[k] = zero;
+    if (!zeta_of(code)) {
+#pragma unroll
+        for (int i = 1; i < 9; ++i) P.g[i * plane + k] = zero;
+        P.g0[k] = T::g0_from_double(0.0);
+        sprev[k] = C(0);
+        return;
+    }
+    // the pull at x + c_j reads this value as its g_j when x + c_j is a zeta = 1
+    // node; when it is not, only the doubly-unknown rule of this node reads
+    // it, as the node's own value
+    const int ty = threadIdx.y, tx = threadIdx.x;
+    double rsum = 0.0;
+#pragma unroll
     for (int j = 1; j < 9; ++j) {
-        int yy = y + cy(j);
-        if (yy < 0 || yy >= ny) continue;
-        size_t m = (size_t)yy * pitch + wrap1(x + cx(j), nx);
-        if (zeta_of(cls[m])) { num += phi[m]; den += 1.0; }
+        const bool z = zeta_of(s_cls[ty + 3 + cy(j)][tx + 3 + cx(j)]);
+        const int r = ty + 1 + (z ? cy(j) : 0), c1 = tx + 1 + (z ? cx(j) : 0), d = j <= 4 ? 0 : 1;
+        const C v = s_g[d][r][c1];
+        P.g[j * plane + k] = j <= 4 ? T::template st<1>(v) : T::template st<5>(v);
+        if constexpr (T::kAbsorb) {
+            const double e = s_res[d][r][c1];
+            if (__double_as_longlong(e) != 0) rsum += e;
+        }
     }
-    phi[k] = num / den;
-}
-
-template <typename C>
-__global__ void k_init_mu(const uint8_t* __restrict__ cls, const C* __restrict__ wet, const double* __restrict__ phi,
-                          double* __restrict__ mu, C* __restrict__ sprev, int nx, int ny, int pitch, Params q)
-{
-    int x = blockIdx.x * blockDim.x + threadIdx.x;
-    int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= nx || y >= ny) return;
-    size_t k = (size_t)y * pitch + x;
-    uint8_t code = cls[k];
-    if (!zeta_of(code)) { mu[k] = 0.0; sprev[k] = (C)0; return; }
-    // in the precision of the step's arithmetic (C): FP64 for FP64 solves,
-    // FP32 otherwise (FP64 arithmetic is slow on this part, and a 32-bit
-    // state stores mu only through g_i^eq = w_i alpha mu, rounded to 32 or
-    // 16 bits; phi = sum g_i stays exact through g_0)
-    auto at = [&](int dx, int dy) { return (C)phi[(size_t)(y + dy) * pitch + wrap1(x + dx, nx)]; };
-    const C c = (C)phi[k];
-    const C E = at(1, 0), Wv = at(-1, 0), N = at(0, 1), S = at(0, -1);
-    const C NE = at(1, 1), NW = at(-1, 1), SW = at(-1, -1), SE = at(1, -1);
-    // multiplications by rounded reciprocals: division is slow
-    const C gpx = (E - Wv) * (C(1) / C(3)) + ((NE + SE) - (NW + SW)) * (C(1) / C(12));
-    const C gpy = (N - S) * (C(1) / C(3)) + ((NE + NW) - (SE + SW)) * (C(1) / C(12));
-    const C lap = ((E + Wv) + (N + S)) * (C(2) / C(3)) + ((NE + NW) + (SE + SW)) * (C(1) / C(6)) - c * (C(10) / C(3));
-    const C wv = (code & F_WET) ? wet[k] : C(0);
-    const C m = C(4) * (C)q.beta * c * (c - C(1)) * (c - C(0.5)) - (C)q.kappa * lap - wv * (c - c * c);
-    mu[k] = (double)m;
-    // u at t = 0 from f = 0: u = F / (2 rho), F = mu grad(phi) + rho g; the
-    // history of the first step is u.grad(phi)
-    const C rho = (C)q.rho_g + (C)(q.rho_l - q.rho_g) * c;
-    const C half_inv_rho = C(0.5) / rho;
-    const C ux = (m * gpx + rho * (C)q.gx) * half_inv_rho, uy = (m * gpy + rho * (C)q.gy) * half_inv_rho;
-    sprev[k] = ux * gpx + uy * gpy;
-}
-
-// g_J^eq (J != 0) in storage form; returns the rounding residual.
-template <int PREC, int J>
-__device__ __forceinline__ double init_g_dir(const uint8_t* cls, const double* mu, const Planes<PREC>& P, int x,
-                                             int y, int nx, int pitch, size_t k, size_t plane, double alpha)
-{
-    using T = Store<PREC>;
-    // the pull at x + c_j reads this value as its g_j when x + c_j is a
-    // zeta = 1 node; when it is not, only the doubly-unknown rule of this
-    // node reads it, as the node's own value
-    size_t m = (size_t)(y + cy(J)) * pitch + wrap1(x + cx(J), nx);
-    if (!zeta_of(cls[m])) m = k;
-    const double w = J <= 4 ? 1.0 / 9.0 : 1.0 / 36.0;
-    const double v = w * alpha * mu[m];
-    const typename T::S s = T::template st<J>((typename T::C)v);
-    P.g[J * plane + k] = s;
-    return v - (double)T::template ld<J>(s);
-}
-
-// Post-collision arrays that the first pull turns into f = 0, g = g^eq(phi0, mu0).
-template <int PREC>
-__global__ void k_init_pop(const uint8_t* __restrict__ cls, const double* __restrict__ phi,
-                           const double* __restrict__ mu, Planes<PREC> P, int nx, int ny, int pitch, size_t plane,
-                           double alpha)
-{
-    using T = Store<PREC>;
-    int x = blockIdx.x * blockDim.x + threadIdx.x;
-    int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= nx || y >= ny) return;
-    size_t k = (size_t)y * pitch + x;
-    const typename T::S zero = T::template st<0>((typename T::C)0);
-    for (int i = 0; i < 9; ++i) {
-        P.f[i * plane + k] = zero;
-        P.g[i * plane + k] = zero;
-    }
-    P.g0[k] = T::g0_from_double(0.0);
-    if (!zeta_of(cls[k])) return;
-    double r = 0.0;
-    r += init_g_dir<PREC, 1>(cls, mu, P, x, y, nx, pitch, k, plane, alpha);
-    r += init_g_dir<PREC, 2>(cls, mu, P, x, y, nx, pitch, k, plane, alpha);
-    r += init_g_dir<PREC, 3>(cls, mu, P, x, y, nx, pitch, k, plane, alpha);
-    r += init_g_dir<PREC, 4>(cls, mu, P, x, y, nx, pitch, k, plane, alpha);
-    r += init_g_dir<PREC, 5>(cls, mu, P, x, y, nx, pitch, k, plane, alpha);
-    r += init_g_dir<PREC, 6>(cls, mu, P, x, y, nx, pitch, k, plane, alpha);
-    r += init_g_dir<PREC, 7>(cls, mu, P, x, y, nx, pitch, k, plane, alpha);
-    r += init_g_dir<PREC, 8>(cls, mu, P, x, y, nx, pitch, k, plane, alpha);
     // g_0^eq (Eq. H_i); with 16-bit g_i it also holds their rounding residual
-    double g0 = phi[k] - (5.0 / 9.0) * alpha * mu[k];
-    if (T::kAbsorb) g0 += r;
-    P.g0[k] = T::g0_from_double(g0);
+    const double ph = s_phi[ty + 3][tx + 3];
+    double g0 = ph;
+    if (s_mu[ty + 1][tx + 1] != C(0)) g0 = ph - (5.0 / 9.0) * q.alpha * (double)s_mu[ty + 1][tx + 1];
+    if (T::kAbsorb && __double_as_longlong(rsum) != 0) g0 += rsum;
+    P.g0[k] = __double_as_longlong(g0) == 0 ? T::g0_from_double(0.0) : T::g0_from_double(g0);
 }
 
 dim3 grid2d(int nx, int ny, dim3 b) { return dim3((nx + b.x - 1) / b.x, (ny + b.y - 1) / b.y); }
@@ -520,15 +584,13 @@ cudaError_t run_step_kernel(pflbm_t* h, double* o_phi, double* o_u, double* o_p,
 }
 
 template <int PREC>
-cudaError_t init_pop_prec(pflbm_t* h)
+cudaError_t init_state_prec(pflbm_t* h)
 {
     using C = typename Store<PREC>::C;
-    dim3 b(32, 8), g = grid2d(h->nx, h->ny, b);
+    dim3 b(TX, TY), g(tiles_x(h->nx), tiles_y(h->ny));
     size_t plane = (size_t)h->ny * h->pitch;
-    k_init_mu<C><<<g, b, 0, h->stream>>>(h->cls, (const C*)h->wet, h->phi0, h->mu0, (C*)h->sprev, h->nx, h->ny,
-                                         h->pitch, h->prm);
-    k_init_pop<PREC><<<g, b, 0, h->stream>>>(h->cls, h->phi0, h->mu0, Planes<PREC>::make(h->pop[h->cur], plane),
-                                             h->nx, h->ny, h->pitch, plane, h->prm.alpha);
+    k_init_state<PREC><<<g, b, 0, h->stream>>>(h->cls, (const C*)h->wet, h->phi0, Planes<PREC>::make(h->pop[h->cur], plane),
+                                               (C*)h->sprev, h->dstatus, h->nx, h->ny, h->pitch, plane, h->prm);
     return cudaGetLastError();
 }
 
@@ -536,43 +598,45 @@ cudaError_t init_pop_prec(pflbm_t* h)
 
 cudaError_t launch_init_phi_droplet(pflbm_t* h, double x0, double y0, double R, int replace)
 {
-    // Outside r = R + 10 W the profile is exactly 0 in FP64 (tanh(-20) rounds
-    // to -1), so only the droplet's bounding box is evaluated; a replacing
-    // call clears the field first.
-    if (replace) {
+    // Beyond `reach` the profile is exactly 0, so only the droplet's bounding
+    // box is evaluated; a replacing call clears the field first.
+    if (replace) h->phi0_nonneg = true;
+    const double reach = droplet_reach(h->precision == PFLBM_FP64, h->phi0_nonneg, R, h->prm.W);
+    int ylo = (int)fmax(0.0, floor(y0 - reach)), yhi = (int)fmin((double)h->ny - 1, ceil(y0 + reach));
+    int xlo = 0, xw = h->nx;
+    // a replacing call clears what its box does not cover; up to this many
+    // nodes the box is the whole lattice instead (the extra nodes cost less than
+    // a second launch: 256 x 128 nodes are 128 CTAs)
+    const bool whole = replace && (long long)h->nx * h->ny <= (1 << 17);
+    if (replace && !whole) {
         cudaError_t e = cudaMemsetAsync(h->phi0, 0, (size_t)h->ny * h->pitch * sizeof(double), h->stream);
         if (e != cudaSuccess) return e;
     }
-    double reach = fabs(R) + 10.0 * h->prm.W;
-    int ylo = (int)fmax(0.0, floor(y0 - reach)), yhi = (int)fmin((double)h->ny - 1, ceil(y0 + reach));
-    if (ylo > yhi) return cudaSuccess;
-    int xlo = 0, xw = h->nx;
-    if (2.0 * reach + 2.0 < h->nx) {
+    if (whole) {
+        ylo = 0;
+        yhi = h->ny - 1;
+    } else if (ylo > yhi) {
+        return cudaSuccess;
+    } else if (2.0 * reach + 2.0 < h->nx) {
         xlo = (int)floor(x0 - reach);
         xw = (int)(ceil(x0 + reach) - floor(x0 - reach)) + 1;
     }
     dim3 b(32, 8), g = grid2d(xw, yhi - ylo + 1, b);
-    if (h->precision == PFLBM_FP64)
-        k_init_droplet<false><<<g, b, 0, h->stream>>>(h->cls, h->phi0, h->nx, h->ny, h->pitch, xlo, xw, ylo, yhi + 1,
-                                                      x0, y0, R, h->prm.W);
-    else
-        k_init_droplet<true><<<g, b, 0, h->stream>>>(h->cls, h->phi0, h->nx, h->ny, h->pitch, xlo, xw, ylo, yhi + 1,
-                                                     x0, y0, R, h->prm.W);
+    auto launch = [&](auto* k) {
+        k<<<g, b, 0, h->stream>>>(h->cls, h->phi0, h->nx, h->ny, h->pitch, xlo, xw, ylo, yhi + 1, x0, y0, R, h->prm.W, reach);
+    };
+    if (h->precision == PFLBM_FP64) whole ? launch(k_init_droplet<false, true>) : launch(k_init_droplet<false, false>);
+    else whole ? launch(k_init_droplet<true, true>) : launch(k_init_droplet<true, false>);
     return cudaGetLastError();
 }
 
 cudaError_t launch_init_populations(pflbm_t* h)
 {
-    dim3 b(32, 8), g = grid2d(h->nx, h->ny, b);
-    if (h->precision == PFLBM_FP64)
-        k_ghost_fill<double><<<g, b, 0, h->stream>>>(h->cls, (const double*)h->wet, h->phi0, h->nx, h->ny, h->pitch);
-    else
-        k_ghost_fill<float><<<g, b, 0, h->stream>>>(h->cls, (const float*)h->wet, h->phi0, h->nx, h->ny, h->pitch);
     switch (h->precision) {
-        case PFLBM_FP64: return init_pop_prec<PFLBM_FP64>(h);
-        case PFLBM_FP32: return init_pop_prec<PFLBM_FP32>(h);
-        case PFLBM_BF16: return init_pop_prec<PFLBM_BF16>(h);
-        default: return init_pop_prec<PFLBM_FP16>(h);
+        case PFLBM_FP64: return init_state_prec<PFLBM_FP64>(h);
+        case PFLBM_FP32: return init_state_prec<PFLBM_FP32>(h);
+        case PFLBM_BF16: return init_state_prec<PFLBM_BF16>(h);
+        default: return init_state_prec<PFLBM_FP16>(h);
     }
 }
 
