@@ -251,8 +251,11 @@ int pflbm3d_init_droplet(pflbm3d_t* h, double x0, double y0, double z0, double R
     DeviceGuard g(h->device);
     if (!std::isfinite(x0) || !std::isfinite(y0) || !std::isfinite(z0) || !std::isfinite(R))
         return fail3(PFLBM_EINVAL, "non-finite droplet");
-    if (h->replace_phi) CK3(cudaMemsetAsync(h->phi0, 0, (size_t)h->nz * h->ny * h->pitch * 8, h->stream));
-    const double reach = fabs(R) + 10.0 * h->prm.W;
+    if (h->replace_phi) {
+        CK3(cudaMemsetAsync(h->phi0, 0, (size_t)h->nz * h->ny * h->pitch * 8, h->stream));
+        h->phi0_nonneg = true;
+    }
+    const double reach = droplet_reach(h->precision == PFLBM_FP64, h->phi0_nonneg, R, h->prm.W);
     auto span = [&](double c, int n, int& lo, int& w) {
         lo = 0;
         w = n;
@@ -267,7 +270,7 @@ int pflbm3d_init_droplet(pflbm3d_t* h, double x0, double y0, double z0, double R
     const int zlo = (int)fmin((double)h->nz, fmax(0.0, floor(z0 - reach)));
     const int zhi = (int)fmax(-1.0, fmin((double)h->nz - 1, ceil(z0 + reach)));
     if (zlo <= zhi) {
-        CK3(launch_droplet(h, xlo, xw, ylo, yw, zlo, zhi - zlo + 1, x0, y0, z0, R));
+        CK3(launch_droplet(h, xlo, xw, ylo, yw, zlo, zhi - zlo + 1, x0, y0, z0, R, reach));
     }
     h->replace_phi = false;
     h->init_pending = true;
@@ -283,6 +286,7 @@ int pflbm3d_init_phi(pflbm3d_t* h, const double* phi)
                           cudaMemcpyHostToDevice, h->stream));
     CK3(cudaStreamSynchronize(h->stream));
     h->replace_phi = false;
+    h->phi0_nonneg = false;
     h->init_pending = true;
     h->steps = 0;
     return PFLBM_OK;

@@ -22,7 +22,7 @@ struct pflbm3d {
     void* sprev = nullptr;
     void* phi = nullptr;
     double* phi0 = nullptr;
-    double* mu0 = nullptr;
+    double* mu0 = nullptr;      // g_i^eq (i != 0) of the initial field, in the arithmetic's type
     double* red = nullptr;
     double* out = nullptr;
     float* out_f = nullptr;     // FP32 read-back scratch (5 dense fields), on first use
@@ -37,6 +37,7 @@ struct pflbm3d {
     int fused_zc = 0;           // planes per CTA of the fused step
     int cur = 0;
     bool replace_phi = true, init_pending = false;
+    bool phi0_nonneg = true;    // phi0 holds droplets only
     int64_t steps = 0;
     // optional device allocator (both NULL: cudaMalloc / cudaFree)
     void* (*alloc_fn)(size_t, void*) = nullptr;
@@ -67,7 +68,7 @@ cudaError_t launch_ghost_collect(pflbm3d_t* h, int* count, int* list);
 cudaError_t launch_ghost_flags(pflbm3d_t* h);
 // Eq. initialphi on the bounding box [xlo, xlo + xw) x [ylo, ylo + yw) x [zlo, zlo + zn)
 cudaError_t launch_droplet(pflbm3d_t* h, int xlo, int xw, int ylo, int yw, int zlo, int zn, double x0, double y0,
-                           double z0, double R);
+                           double z0, double R, double reach);
 // shared-memory attribute and resident CTAs per SM of the fused step kernel
 cudaError_t fused_setup(int precision, size_t* smem_bytes, int* ctas_per_sm);
 
