@@ -113,6 +113,33 @@ cudaError_t launch_contact_angle3d(const uint8_t* cls, const double* d_phi, int 
                                    const Wall3& w, double* pts, int cap, int* d_count, double* d_out,
                                    cudaStream_t stream);
 
+// Programmatic dependent launch, for the chains of step kernels: a kernel
+// launched with launch_after may start once every CTA of the one before it in
+// the stream has begun, and waits in step_wait() until that one is complete and
+// its writes are visible. What it does before (node bytes, indexes, prefetches) and
+// its CTAs' start-up overlap the other's last wave. Every CTA calls step_wait()
+// first thing after its static reads, so a kernel that has ended implies that
+// all before it have. Both are no-ops in a plain launch.
+__device__ __forceinline__ void step_wait()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename K, typename... A>
+cudaError_t launch_after(K* kernel, dim3 grid, dim3 block, cudaStream_t stream, const A&... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // Distance from its centre beyond which a droplet's profile 1/2 + 1/2 tanh(2 (R -
 // r) / W) is exactly 0. FP64: |R| + 10 W (tanh(-20) rounds to -1). FP32:
 // |R| + 6 W, since tanhf is exactly -1 at an argument of -12 and beyond (checked

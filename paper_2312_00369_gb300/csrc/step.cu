@@ -278,6 +278,7 @@ __global__ void __launch_bounds__(TX * TY, PREC == PFLBM_FP64 ? 1 : PFLBM_STEP_M
     __shared__ uint8_t s_cls[TY + 6][TX + 6];
     __shared__ typename Store<PREC>::C s_phi[TY + 4][TX + 4];
     if (COLLIDE && PFLBM_L2_AHEAD > 0) prefetch_tile_l2<PREC>(a, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
+    if (COLLIDE) step_wait();
     step_tile<PREC, COLLIDE, VV>(a, blockIdx.x, blockIdx.y, gridDim.x, s_cls, s_phi);
 }
 
@@ -576,11 +577,16 @@ cudaError_t run_step_kernel(pflbm_t* h, double* o_phi, double* o_u, double* o_p,
     a.f_u = f_u;
     a.f_p = f_p;
     dim3 b(TX, TY), g(tiles_x(h->nx), tiles_y(h->ny));
-    if (a.varvisc)
-        k_step<PREC, COLLIDE, 1><<<g, b, 0, h->stream>>>(a);
-    else
-        k_step<PREC, COLLIDE, 0><<<g, b, 0, h->stream>>>(a);
-    return cudaGetLastError();
+    if constexpr (COLLIDE) {
+        return a.varvisc ? launch_after(k_step<PREC, true, 1>, g, b, h->stream, a)
+                         : launch_after(k_step<PREC, true, 0>, g, b, h->stream, a);
+    } else {
+        if (a.varvisc)
+            k_step<PREC, false, 1><<<g, b, 0, h->stream>>>(a);
+        else
+            k_step<PREC, false, 0><<<g, b, 0, h->stream>>>(a);
+        return cudaGetLastError();
+    }
 }
 
 template <int PREC>

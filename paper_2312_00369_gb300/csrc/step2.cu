@@ -582,6 +582,7 @@ __global__ void __launch_bounds__(QTX * QY, PREC == PFLBM_FP32 ? PFLBM_STEP2_MIN
     __shared__ __align__(16) float s_phi[QY + 4][QPW];
     __shared__ uint16_t s_gw[QGP];
     if (PFLBM_L2_AHEAD2 > 0) prefetch2_l2<PREC>(a, blockIdx.x, blockIdx.y);
+    step_wait();
     const int x0 = blockIdx.x * QX;
     // every x the tile touches inside the lattice (the pulls of the second
     // phi ring reach three nodes out)
@@ -654,11 +655,7 @@ cudaError_t run2(pflbm_t* h)
     dim3 b(QTX, QY), g((h->nx + QX - 1) / QX, (h->ny + QY - 1) / QY);
     a.pf_dx = PFLBM_L2_AHEAD2 % (int)g.x;
     a.pf_dy = PFLBM_L2_AHEAD2 / (int)g.x;
-    if (a.varvisc)
-        k_step2<PREC, 1><<<g, b, 0, h->stream>>>(a);
-    else
-        k_step2<PREC, 0><<<g, b, 0, h->stream>>>(a);
-    return cudaGetLastError();
+    return a.varvisc ? launch_after(k_step2<PREC, 1>, g, b, h->stream, a) : launch_after(k_step2<PREC, 0>, g, b, h->stream, a);
 }
 
 }  // namespace

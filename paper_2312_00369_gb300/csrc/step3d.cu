@@ -171,6 +171,7 @@ __global__ void __launch_bounds__(256) k3_phi(Args3<PREC> a)
 {
     using C = typename Store<PREC>::C;
     if (PFLBM3D_PHI_AHEAD > 0) prefetch_phi_rows_l2<PREC>(a);
+    step_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
     if (x >= a.nx || y >= a.ny || z == 0 || z == a.nz - 1) return;
     const int k = (z * a.ny + y) * a.pitch + x;
@@ -190,17 +191,23 @@ __global__ void __launch_bounds__(256) k3_ghost(Args3<PREC> a, const int* __rest
 {
     using C = typename Store<PREC>::C;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n_ghosts) return;
-    const int k = ghosts[t];
+    const bool in = t < n_ghosts;
+    const int k = in ? ghosts[t] : 0;
     const int x = k % a.pitch, y = (k / a.pitch) % a.ny, z = k / (a.pitch * a.ny);
+    // which of the 27 count, read before the wait for phi
+    unsigned zeta = 0;
+#pragma unroll
+    for (int j = 0; j < 27; ++j) {
+        const int dz = j / 9 - 1, dy = j / 3 % 3 - 1, dx = j % 3 - 1;
+        if (in && z + dz >= 0 && z + dz < a.nz && zeta_of(a.cls[nbr(a, x, y, z, dx, dy, dz)])) zeta |= 1u << j;
+    }
+    step_wait();
+    if (!in) return;
     C num = C(0), den = C(0);
-    for (int dz = -1; dz <= 1; ++dz) {
-        if (z + dz < 0 || z + dz >= a.nz) continue;
-        for (int dy = -1; dy <= 1; ++dy)
-            for (int dx = -1; dx <= 1; ++dx) {
-                const int m = nbr(a, x, y, z, dx, dy, dz);
-                if (zeta_of(a.cls[m])) { num += a.phi[m]; den += C(1); }
-            }
+#pragma unroll
+    for (int j = 0; j < 27; ++j) {
+        const int dz = j / 9 - 1, dy = j / 3 % 3 - 1, dx = j % 3 - 1;
+        if (zeta >> j & 1u) { num += a.phi[nbr(a, x, y, z, dx, dy, dz)]; den += C(1); }
     }
     a.phi[k] = num / den;
 }
@@ -355,6 +362,7 @@ __device__ __forceinline__ void step_node(const Args3<PREC>& a, int x, int y, in
 template <int PREC, bool COLLIDE>
 __global__ void __launch_bounds__(256, PREC == PFLBM_FP64 ? 1 : PFLBM3D_STEP_MINB) k3_step(Args3<PREC> a)
 {
+    if (COLLIDE) step_wait();   // (a class byte held over the wait costs spills)
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
     if (x >= a.nx || y >= a.ny) return;
     const int k = (z * a.ny + y) * a.pitch + x;
@@ -913,10 +921,12 @@ cudaError_t step3_prec(pflbm3d_t* h)
         k3_fused<PREC><<<gf, b, fused_smem_bytes<PREC>(), h->stream>>>(a, h->fused_zc, h->gflag);
         return cudaGetLastError();
     }
-    k3_phi<PREC><<<g, b, 0, h->stream>>>(a);
-    if (h->n_ghosts) k3_ghost<PREC><<<(h->n_ghosts + 255) / 256, 256, 0, h->stream>>>(a, h->ghosts, h->n_ghosts);
-    k3_step<PREC, true><<<g, b, 0, h->stream>>>(a);
-    return cudaGetLastError();
+    cudaError_t e = launch_after(k3_phi<PREC>, g, b, h->stream, a);
+    if (e == cudaSuccess && h->n_ghosts)
+        e = launch_after(k3_ghost<PREC>, dim3((h->n_ghosts + 255) / 256), dim3(256), h->stream, a, (const int*)h->ghosts,
+                         h->n_ghosts);
+    if (e == cudaSuccess) e = launch_after(k3_step<PREC, true>, g, b, h->stream, a);
+    return e;
 }
 
 template <int PREC>
