@@ -464,6 +464,7 @@ int pflbm_create_ex(pflbm_t** out, const pflbm_params_t* prm)
     CKR(cudaMemsetAsync(h->phi0, 0, s.N * sizeof(double), h->stream));
     CKR(cudaMemsetAsync(h->solid, 1, s.N, h->stream));
     CKR(cudaMemsetAsync(h->dstatus, 0, sizeof(int) * 4, h->stream));
+    CKR(cudaMemsetAsync(h->red, 0, s.red, h->stream));
     CKR(cudaMemcpy2DAsync(h->solid, h->pitch, prm->solid_mask, nx, nx, ny, cudaMemcpyHostToDevice, h->stream));
     if (prm->theta_field_deg)
         CKR(cudaMemcpy2DAsync(h->theta, h->pitch * sizeof(float), prm->theta_field_deg, nx * sizeof(float),

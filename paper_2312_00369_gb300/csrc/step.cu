@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(TX * TY, PREC == PFLBM_FP64 ? 1 : PFLBM_STEP_M
     __shared__ uint8_t s_cls[TY + 6][TX + 6];
     __shared__ typename Store<PREC>::C s_phi[TY + 4][TX + 4];
     if (COLLIDE && PFLBM_L2_AHEAD > 0) prefetch_tile_l2<PREC>(a, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
-    if (COLLIDE) step_wait();
+    step_wait();
     step_tile<PREC, COLLIDE, VV>(a, blockIdx.x, blockIdx.y, gridDim.x, s_cls, s_phi);
 }
 
@@ -359,6 +359,23 @@ StepArgs<PREC> make_args(pflbm_t* h)
 // ---------------------------------------------------------------------------
 // Initial state (FP64 arithmetic for every storage precision)
 // ---------------------------------------------------------------------------
+// 1/2 + 1/2 tanh(2 (R - r) / W) at node (x, y), r periodic in x (Eq.
+// initialphi); 0 beyond `reach` (droplet_reach).
+template <bool F32>
+__device__ __forceinline__ double droplet_profile(int x, int y, int nx, double x0, double y0, double R, double W,
+                                                  double reach)
+{
+    double dx = fabs((double)x - x0);
+    if (dx >= nx) dx = fmod(dx, (double)nx);   // exact; only for a period or more
+    if (dx > 0.5 * nx) dx = nx - dx;           // x-periodic distance
+    const double dy = (double)y - y0, r2 = dx * dx + dy * dy;
+    // beyond `reach` the profile is 0 (droplet_reach): the bounding box's
+    // corners are skipped like the nodes outside it
+    if (r2 > reach * reach) return 0.0;
+    return F32 ? (double)(0.5f + 0.5f * tanhf(2.0f * ((float)R - sqrtf((float)r2)) / (float)W))
+                         : 0.5 + 0.5 * tanh(2.0 * (R - sqrt(r2)) / W);
+}
+
 // Eq. initialphi over the box x in [xlo, xlo + xw) (x periodic), y in
 // [ylo, yhi), combined with the field by maximum (a replacing call cleared it).
 // F32: the profile in FP32 (solves whose arithmetic is FP32 or 16-bit storage;
@@ -370,24 +387,18 @@ __global__ void k_init_droplet(const uint8_t* __restrict__ cls, double* __restri
                                int pitch, int xlo, int xw, int ylo, int yhi, double x0, double y0, double R,
                                double W, double reach)
 {
+    // the profile does not depend on the field: it is evaluated before the wait
+    // for the droplet before this one
+    double v = 0.0;
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     int y = ylo + blockIdx.y * blockDim.y + threadIdx.y;
-    if (i >= xw || y >= yhi) return;
+    const bool in = i < xw && y < yhi;
     int x = (xlo + i) % nx;
     if (x < 0) x += nx;
-    size_t k = (size_t)y * pitch + x;
-    if (REPLACE) phi[k] = 0.0;
-    if (!zeta_of(cls[k])) return;
-    double dx = fabs((double)x - x0);
-    if (dx >= nx) dx = fmod(dx, (double)nx);   // exact; only for a period or more
-    if (dx > 0.5 * nx) dx = nx - dx;           // x-periodic distance
-    const double dy = (double)y - y0, r2 = dx * dx + dy * dy;
-    // beyond `reach` the profile is 0 (droplet_reach): the bounding box's
-    // corners are skipped like the nodes outside it
-    if (r2 > reach * reach) return;
-    const double v = F32 ? (double)(0.5f + 0.5f * tanhf(2.0f * ((float)R - sqrtf((float)r2)) / (float)W))
-                         : 0.5 + 0.5 * tanh(2.0 * (R - sqrt(r2)) / W);
-    if (REPLACE || v > phi[k]) phi[k] = v;
+    const size_t k = (size_t)y * pitch + x;
+    if (in && zeta_of(cls[k])) v = droplet_profile<F32>(x, y, nx, x0, y0, R, W, reach);
+    step_wait();
+    if (in && (REPLACE || v > phi[k])) phi[k] = v;
 }
 
 // The initial state in one pass: ghost values of phi0 (Sec. 2.2.2), mu of the
@@ -428,6 +439,7 @@ __global__ void __launch_bounds__(TX * TY) k_init_state(const uint8_t* __restric
     __shared__ double s_res[T::kAbsorb ? 2 : 1][H1][W1];     // and what storage rounds off them
     const int tid = threadIdx.y * TX + threadIdx.x;
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    step_wait();
     if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *status = 0;
 
     bool phase = false;
@@ -577,16 +589,8 @@ cudaError_t run_step_kernel(pflbm_t* h, double* o_phi, double* o_u, double* o_p,
     a.f_u = f_u;
     a.f_p = f_p;
     dim3 b(TX, TY), g(tiles_x(h->nx), tiles_y(h->ny));
-    if constexpr (COLLIDE) {
-        return a.varvisc ? launch_after(k_step<PREC, true, 1>, g, b, h->stream, a)
-                         : launch_after(k_step<PREC, true, 0>, g, b, h->stream, a);
-    } else {
-        if (a.varvisc)
-            k_step<PREC, false, 1><<<g, b, 0, h->stream>>>(a);
-        else
-            k_step<PREC, false, 0><<<g, b, 0, h->stream>>>(a);
-        return cudaGetLastError();
-    }
+    return a.varvisc ? launch_after(k_step<PREC, COLLIDE, 1>, g, b, h->stream, a)
+                     : launch_after(k_step<PREC, COLLIDE, 0>, g, b, h->stream, a);
 }
 
 template <int PREC>
@@ -595,9 +599,9 @@ cudaError_t init_state_prec(pflbm_t* h)
     using C = typename Store<PREC>::C;
     dim3 b(TX, TY), g(tiles_x(h->nx), tiles_y(h->ny));
     size_t plane = (size_t)h->ny * h->pitch;
-    k_init_state<PREC><<<g, b, 0, h->stream>>>(h->cls, (const C*)h->wet, h->phi0, Planes<PREC>::make(h->pop[h->cur], plane),
-                                               (C*)h->sprev, h->dstatus, h->nx, h->ny, h->pitch, plane, h->prm);
-    return cudaGetLastError();
+    return launch_after(k_init_state<PREC>, g, b, h->stream, (const uint8_t*)h->cls, (const C*)h->wet,
+                        (const double*)h->phi0, Planes<PREC>::make(h->pop[h->cur], plane), (C*)h->sprev, h->dstatus, h->nx,
+                        h->ny, h->pitch, plane, h->prm);
 }
 
 }  // namespace
@@ -629,11 +633,12 @@ cudaError_t launch_init_phi_droplet(pflbm_t* h, double x0, double y0, double R, 
     }
     dim3 b(32, 8), g = grid2d(xw, yhi - ylo + 1, b);
     auto launch = [&](auto* k) {
-        k<<<g, b, 0, h->stream>>>(h->cls, h->phi0, h->nx, h->ny, h->pitch, xlo, xw, ylo, yhi + 1, x0, y0, R, h->prm.W, reach);
+        return launch_after(k, g, b, h->stream, (const uint8_t*)h->cls, h->phi0, h->nx, h->ny, h->pitch, xlo, xw, ylo, yhi + 1,
+                            x0, y0, R, h->prm.W, reach);
     };
-    if (h->precision == PFLBM_FP64) whole ? launch(k_init_droplet<false, true>) : launch(k_init_droplet<false, false>);
-    else whole ? launch(k_init_droplet<true, true>) : launch(k_init_droplet<true, false>);
-    return cudaGetLastError();
+    if (h->precision == PFLBM_FP64)
+        return whole ? launch(k_init_droplet<false, true>) : launch(k_init_droplet<false, false>);
+    return whole ? launch(k_init_droplet<true, true>) : launch(k_init_droplet<true, false>);
 }
 
 cudaError_t launch_init_populations(pflbm_t* h)

@@ -362,7 +362,7 @@ __device__ __forceinline__ void step_node(const Args3<PREC>& a, int x, int y, in
 template <int PREC, bool COLLIDE>
 __global__ void __launch_bounds__(256, PREC == PFLBM_FP64 ? 1 : PFLBM3D_STEP_MINB) k3_step(Args3<PREC> a)
 {
-    if (COLLIDE) step_wait();   // (a class byte held over the wait costs spills)
+    step_wait();   // (a class byte held over the wait costs spills)
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
     if (x >= a.nx || y >= a.ny) return;
     const int k = (z * a.ny + y) * a.pitch + x;
@@ -706,6 +706,7 @@ __global__ void __launch_bounds__(256) k3_droplet(const uint8_t* __restrict__ cl
         s_z2[tid - 40] = d * d;
     }
     __syncthreads();
+    step_wait();
     const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y;
     if (i >= xw || j >= yw) return;
     const size_t col = (size_t)node(ylo + j, ny) * pitch + node(xlo + i, nx);
@@ -941,10 +942,12 @@ cudaError_t macro3_prec(pflbm3d_t* h, double* phi, double* u, double* p, float* 
     a.f_u = fu;
     a.f_p = fp;
     dim3 b(32, 8), g = grid3(h);
-    k3_phi<PREC><<<g, b, 0, h->stream>>>(a);
-    if (h->n_ghosts) k3_ghost<PREC><<<(h->n_ghosts + 255) / 256, 256, 0, h->stream>>>(a, h->ghosts, h->n_ghosts);
-    k3_step<PREC, false><<<g, b, 0, h->stream>>>(a);
-    return cudaGetLastError();
+    cudaError_t e = launch_after(k3_phi<PREC>, g, b, h->stream, a);
+    if (e == cudaSuccess && h->n_ghosts)
+        e = launch_after(k3_ghost<PREC>, dim3((h->n_ghosts + 255) / 256), dim3(256), h->stream, a, (const int*)h->ghosts,
+                         h->n_ghosts);
+    if (e == cudaSuccess) e = launch_after(k3_step<PREC, false>, g, b, h->stream, a);
+    return e;
 }
 
 template <int PREC>
@@ -1037,9 +1040,8 @@ cudaError_t launch_droplet(pflbm3d_t* h, int xlo, int xw, int ylo, int yw, int z
 {
     dim3 b(32, 8), g((xw + 31) / 32, (yw + 7) / 8, (zn + kDropZ - 1) / kDropZ);
     auto* k = h->precision == PFLBM_FP64 ? k3_droplet<false> : k3_droplet<true>;
-    k<<<g, b, 0, h->stream>>>(h->cls, h->phi0, h->nx, h->ny, h->pitch, xlo, xw, ylo, yw, zlo, zn, x0, y0, z0, R, h->prm.W,
-                              reach);
-    return cudaGetLastError();
+    return launch_after(k, g, b, h->stream, (const uint8_t*)h->cls, h->phi0, h->nx, h->ny, h->pitch, xlo, xw, ylo, yw, zlo, zn,
+                        x0, y0, z0, R, h->prm.W, reach);
 }
 
 cudaError_t fused_setup(int precision, size_t* smem_bytes, int* ctas_per_sm)
