@@ -312,12 +312,17 @@ __device__ __forceinline__ void stencils(const C (*s_phi)[PW], int py, int px, C
                 lap);
 }
 
+// What a lane collides and stores (kParts): by default all of it. Warps that
+// share a node take a part each; all of them evaluate the moments.
+constexpr int kPartAxes = 1, kPartDiagonals = 2, kPartG = 4, kPartAll = 7;
+
 // One node per thread, stored at index k.
 template <int PREC>
 struct Lane1 {
     using T = Store<PREC>;
     using C = typename T::C;
     using FArr = C[9];
+    static constexpr int kParts = kPartAll;
     uint8_t code;
     int k;
     typename T::G0T g0raw;
@@ -406,6 +411,7 @@ struct Lane2 {
     using T = Store<PREC>;
     using C = F2;
     static_assert(PREC != PFLBM_FP64, "packed lanes are FP32");
+    static constexpr int kParts = kPartAll;
     uint8_t code[2];
     bool valid[2];
     int k;
@@ -576,7 +582,7 @@ __device__ __forceinline__ void node_core(const StepArgs<PREC>& a, const L& lane
         readback(ph, ux, uy, p);
         return;
     } else {
-        lane.check_u(a, uu);
+        if constexpr ((L::kParts & kPartG) != 0) lane.check_u(a, uu);
         // relaxation of f: uniform, or tau_f(x) = nu(phi) / c_s^2 + 1/2 with
         // nu(phi) = phi (nu_l - nu_g) + nu_g (Secs. 2.1.1, 2.1.2)
         C omega_f = C(a.omega_f), force_pre = C(a.force_pre);
@@ -586,14 +592,14 @@ __device__ __forceinline__ void node_core(const StepArgs<PREC>& a, const L& lane
         }
 
         // ---- f collision: f* = f + (f^eq - f)/tau_f + F_i ----
-        {
+        if constexpr ((L::kParts & kPartAxes) != 0) {
             const C feq0 = fmadd(-(rho * C(wgt<R>(0) * R(1.5))), uu, C(R(-5) / R(3)) * p);
             C d0f;
             if constexpr (T::kNorm) d0f = fmadd(feq0, C(R(1) / T::template unit<0>()), -f[0]);
             else d0f = feq0 - f[0];
             lane.template store_f<0>(a, fmadd(omega_f, d0f, f[0]));
         }
-        {
+        if constexpr ((L::kParts & (kPartAxes | kPartDiagonals)) != 0) {
             PairK<C> K;
             K.base = omega_f * fmadd(-(C(1.5) * rho), uu, C(3) * p);
             K.c45 = omega_f * C(4.5) * rho;
@@ -606,11 +612,16 @@ __device__ __forceinline__ void node_core(const StepArgs<PREC>& a, const L& lane
                 K.c3 = K.c3 * C(T::scale());
                 K.pre3 = K.pre3 * C(T::scale());
             }
-            collide_f_pair<PREC, 1, 3>(a, lane, f[1], f[3], K, ux, uy, Fx, Fy, drx, dry);
-            collide_f_pair<PREC, 2, 4>(a, lane, f[2], f[4], K, ux, uy, Fx, Fy, drx, dry);
-            collide_f_pair<PREC, 5, 7>(a, lane, f[5], f[7], K, ux, uy, Fx, Fy, drx, dry);
-            collide_f_pair<PREC, 6, 8>(a, lane, f[6], f[8], K, ux, uy, Fx, Fy, drx, dry);
+            if constexpr ((L::kParts & kPartAxes) != 0) {
+                collide_f_pair<PREC, 1, 3>(a, lane, f[1], f[3], K, ux, uy, Fx, Fy, drx, dry);
+                collide_f_pair<PREC, 2, 4>(a, lane, f[2], f[4], K, ux, uy, Fx, Fy, drx, dry);
+            }
+            if constexpr ((L::kParts & kPartDiagonals) != 0) {
+                collide_f_pair<PREC, 5, 7>(a, lane, f[5], f[7], K, ux, uy, Fx, Fy, drx, dry);
+                collide_f_pair<PREC, 6, 8>(a, lane, f[6], f[8], K, ux, uy, Fx, Fy, drx, dry);
+            }
         }
+        if constexpr ((L::kParts & kPartG) == 0) return;
 
         // ---- g collision: g* = g + (g^eq - g)/tau_g + (3/2) G_i(t) - (1/2) G_i(t-1) ----
         const C s_now = fmadd(ux, gpx, uy * gpy);
