@@ -320,10 +320,19 @@ def batched_line(args, torch, world, local, steps, warmup, plain=True, precision
         "plain_fp32_one_launch_per_lattice_mlups": plain_mlups,
         "speedup_vs_plain": (value / plain_mlups) if plain_mlups else None,
         "autotune_ms_per_step": timings,
-        # the two-node batched kernel runs one launch per group of same-size
-        # lattices each step (batch info's grid); the others one launch
-        "gpu_launches": (info["grid"] if kernel == 3 else 1) * steps, "clocks": clocks,
+        "gpu_launches": batched_launches(kernel, info["grid"], nodes, steps), "clocks": clocks,
     }
+
+
+def batched_launches(kernel, grid, nodes, steps):
+    """Step kernels launched by a batched run, at least. The two-node kernel
+    runs one launch per group of same-size lattices each step (batch info's
+    grid), the others one launch a step. Runs of 16 steps and more may go
+    through the resident kernel instead: waves of at most 152 patches of at
+    most 2048 nodes, each wave one launch per 1024 steps."""
+    if kernel == 2 or steps < 16:
+        return (grid if kernel == 3 else 1) * steps
+    return -(-nodes // (152 * 2048)) * -(-steps // 1024)
 
 
 def run_serving(args, torch, rank, world, local):

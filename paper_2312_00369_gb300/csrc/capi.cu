@@ -202,12 +202,14 @@ int ensure_out(pflbm_t* h)
 }
 
 // Step kernel of a handle (pflbm_params_t.step_kernel). 0 picks the default
-// by storage and lattice size, from the measured crossover on lattices of 5k
-// to 8.4M nodes (warm, MLUPS):
-// - 16-bit storage: the two-node kernel from 2^19 nodes (6 to 32 % faster
-//   there; 5 to 25 % slower at 2^18 nodes and below);
-// - FP32: the two-node kernel from 2^21 nodes (2 to 4 % faster there; within
-//   0.5 % at 2^20 nodes, 0.2 to 25 % slower at 2^19 nodes and below);
+// by storage and lattice size, from the measured crossover on lattices of 33k
+// to 8.4M nodes (warm, us a step, one-node and two-node kernel):
+// - 16-bit storage: the two-node kernel from 2^19 nodes (14.0 and 13.7 there,
+//   43.9 and 37.8 at 2^21, 165 and 123 at 2^23; at 409,600 nodes 12.0 and
+//   12.4, at 2^15 5.7 and 7.2);
+// - FP32: the two-node kernel from 2^21 nodes (55.0 and 52.6 there, 195 and 187
+//   at 2^23; within 1.5 % from 2^19 to 1.6M nodes; at 409,600 nodes 11.8 and
+//   12.4, at 2^15 5.8 and 6.8);
 // - otherwise, and for FP64, the one-node global-load kernel: its 32 x 8
 //   tiles give a small lattice twice the CTAs, and each CTA does half the
 //   work. The staged kernel was slower on every workload (about 6 % more
@@ -240,8 +242,11 @@ int select_step_kernel(pflbm_t* h, int kernel, int chunk)
 
 // Runs of at least this many steps are taken resident where the lattice fits
 // (resident.cu), when the step kernel is the library's choice. A resident
-// launch costs about 15 us more than a step's (cooperative launch, loading
-// the state, its lists), and saves 3 to 5 us a step: even at 4 to 5 steps.
+// launch takes 16 to 60 us before its first step (cooperative launch, loading
+// the state, its lists). Measured, 16 single steps and 16 resident (us): FP32
+// 100 x 50 82 and 50, 256 x 128 92 and 66, 400 x 200 106 and 98, 512 x 512 155 and
+// 159 (at 32 steps 310 and 253); BF16 512 x 512 159 and 127; FP64 100 x 50 300
+// and 123, 256 x 128 271 and 247.
 constexpr int64_t kResidentMinSteps = 16;
 constexpr int kResidentMaxSteps = 1024;          // steps of one launch: a few milliseconds
 constexpr long long kResidentMapNodes = 1 << 20; // larger lattices never fit

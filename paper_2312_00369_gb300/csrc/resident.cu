@@ -8,10 +8,11 @@
 // shared memory for all the steps, and after each step the CTAs exchange what
 // their neighbours' pulls reach.
 //
-// Measured (us per step in runs of 1000, one launch per step -> resident):
-// FP32 100 x 50 6.16 -> 2.35, 256 x 128 6.17 -> 2.53, 400 x 200 with a 30 degree
-// slope 8.21 -> 2.84, 512 x 512 with a disc 10.3 -> 6.1 (BF16 10.7 -> 4.9);
-// FP64 100 x 50 18.4 -> 8.0, 400 x 200 41.0 -> 18.2. What a step of 256 x 128
+// Measured (us per step in runs of 1000, one launch per step -> resident; the
+// launches in brackets overlap their heads and tails, launch_after):
+// FP32 100 x 50 6.16 (5.1) -> 2.04, 256 x 128 6.17 (5.8) -> 2.42, 400 x 200 with
+// a 30 degree slope 8.21 (6.6) -> 2.83, 512 x 512 with a disc 10.3 (9.7) -> 5.9
+// (BF16 10.7 (9.9) -> 5.0); FP64 100 x 50 18.4 -> 6.1, 400 x 200 41.0 -> 18.2. What a step of 256 x 128
 // takes (cycles, a patch at the wall): bounce-back copies, pulls and phi
 // 1,100, ghost values 800, collision 1,000, publishing 400, the wait 1,650. With
 // larger patches the pulls (shared-memory bandwidth) and the collision (FP32

@@ -357,7 +357,8 @@ StepArgs<PREC> make_args(pflbm_t* h)
 }
 
 // ---------------------------------------------------------------------------
-// Initial state (FP64 arithmetic for every storage precision)
+// Initial state: phi and g_0 in FP64 for every storage precision; mu and the other
+// populations, which are 0 away from the interfaces, in the step's arithmetic type
 // ---------------------------------------------------------------------------
 // 1/2 + 1/2 tanh(2 (R - r) / W) at node (x, y), r periodic in x (Eq.
 // initialphi); 0 beyond `reach` (droplet_reach).
