@@ -49,6 +49,23 @@
 namespace pfk {
 namespace {
 
+// Whether a lattice's next step takes its tile rows from the last down (DOWN):
+// k_step takes the rows of larger FP32 lattices up and down in turn (the copy
+// read says which), so that a step begins with what L2 (129 MB) still holds of
+// the rows written last. Measured, us a step (in brackets what a step reads and
+// writes), always up and in turn: 1021 x 383 (59 MB) 11.6 and 11.9, 1024 x 768
+// (120 MB) 24.6 and 22.4, 1024 x 1024 (159 MB) 31.8 and 29.0, 1500 x 1000 (228 MB) 40.5
+// and 38.8. From 2^21 nodes k_step2 is the default. The direction is a template
+// argument: read from the descriptor it cost the other lattices 0.5 to 1 %.
+// (k_step2 with it as a template argument lost 3 to 12 %, the overlap of its
+// launches; read from the descriptor it gained 0.5 to 11 % where L2 holds a part
+// and lost 0.5 % at 4096 x 2048 in BF16.)
+bool rows_down(const pflbm_t* h)
+{
+    const double nodes = (double)h->nx * h->ny;
+    return h->cur && h->precision == PFLBM_FP32 && 152.0 * nodes > 64e6 && nodes < (double)(1 << 21);
+}
+
 // Prologue of a tile whose nodes within two of it are all fluid: no class
 // tile, no bounce-back checks, no ghosts, phi on a one-node ring.
 template <int PREC, bool WRAP>
@@ -246,7 +263,7 @@ __device__ __forceinline__ void step_tile(const StepArgs<PREC>& a, int bx, int b
 // multiple of 32 and the pitch of 64). Every address lies inside the
 // lattice's arrays: the tile exists and y < ny; offsets stay below
 // 18 * plane < 2^31.
-template <int PREC>
+template <int PREC, bool DOWN>
 __device__ __forceinline__ void prefetch_tile_l2(const StepArgs<PREC>& a, int bx, int by, int ntx, int nty)
 {
     static_assert(TY == 8, "one row of the tile per thread of an 8-thread group");
@@ -254,6 +271,8 @@ __device__ __forceinline__ void prefetch_tile_l2(const StepArgs<PREC>& a, int bx
     int px = bx + a.pf_dx, py = by + a.pf_dy;
     if (px >= ntx) { px -= ntx; ++py; }
     const int tid = threadIdx.y * TX + threadIdx.x;
+    if (DOWN && py >= nty) return;
+    if (DOWN) py = nty - 1 - py;
     const int q = tid >> 3, gy = py * TY + (tid & 7);
     if (py >= nty || q >= 20 || gy >= a.ny) return;
     const int row = gy * a.pitch + px * TX;
@@ -272,14 +291,14 @@ __device__ __forceinline__ void prefetch_tile_l2(const StepArgs<PREC>& a, int bx
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
-template <int PREC, bool COLLIDE, int VV>
+template <int PREC, bool COLLIDE, int VV, bool DOWN = false>
 __global__ void __launch_bounds__(TX * TY, PREC == PFLBM_FP64 ? 1 : PFLBM_STEP_MINB) k_step(StepArgs<PREC> a)
 {
     __shared__ uint8_t s_cls[TY + 6][TX + 6];
     __shared__ typename Store<PREC>::C s_phi[TY + 4][TX + 4];
-    if (COLLIDE && PFLBM_L2_AHEAD > 0) prefetch_tile_l2<PREC>(a, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
+    if (COLLIDE && PFLBM_L2_AHEAD > 0) prefetch_tile_l2<PREC, DOWN>(a, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
     step_wait();
-    step_tile<PREC, COLLIDE, VV>(a, blockIdx.x, blockIdx.y, gridDim.x, s_cls, s_phi);
+    step_tile<PREC, COLLIDE, VV>(a, blockIdx.x, DOWN ? gridDim.y - 1 - blockIdx.y : blockIdx.y, gridDim.x, s_cls, s_phi);
 }
 
 // Persistent step over many lattices: work item w = (instance, first tile);
@@ -600,6 +619,11 @@ cudaError_t run_step_kernel(pflbm_t* h, double* o_phi, double* o_u, double* o_p,
         else
             k_step<PREC, COLLIDE, 0><<<g, b, 0, h->stream>>>(a);
         return cudaGetLastError();
+    }
+    if constexpr (COLLIDE && PREC == PFLBM_FP32) {
+        if (rows_down(h))
+            return a.varvisc ? launch_after(k_step<PREC, COLLIDE, 1, true>, g, b, h->stream, a)
+                             : launch_after(k_step<PREC, COLLIDE, 0, true>, g, b, h->stream, a);
     }
     return a.varvisc ? launch_after(k_step<PREC, COLLIDE, 1>, g, b, h->stream, a)
                      : launch_after(k_step<PREC, COLLIDE, 0>, g, b, h->stream, a);
