@@ -380,7 +380,8 @@ StepArgs<PREC> make_args(pflbm_t* h)
 // populations, which are 0 away from the interfaces, in the step's arithmetic type
 // ---------------------------------------------------------------------------
 // 1/2 + 1/2 tanh(2 (R - r) / W) at node (x, y), r periodic in x (Eq.
-// initialphi); 0 beyond `reach` (droplet_reach).
+// initialphi). Beyond `reach` (droplet_reach) a node is not the droplet's: -inf,
+// which never wins the maximum with the field.
 template <bool F32>
 __device__ __forceinline__ double droplet_profile(int x, int y, int nx, double x0, double y0, double R, double W,
                                                   double reach)
@@ -389,9 +390,8 @@ __device__ __forceinline__ double droplet_profile(int x, int y, int nx, double x
     if (dx >= nx) dx = fmod(dx, (double)nx);   // exact; only for a period or more
     if (dx > 0.5 * nx) dx = nx - dx;           // x-periodic distance
     const double dy = (double)y - y0, r2 = dx * dx + dy * dy;
-    // beyond `reach` the profile is 0 (droplet_reach): the bounding box's
-    // corners are skipped like the nodes outside it
-    if (r2 > reach * reach) return 0.0;
+    // the bounding box's corners are left alone like the nodes outside it
+    if (r2 > reach * reach) return -INFINITY;
     return F32 ? (double)(0.5f + 0.5f * tanhf(2.0f * ((float)R - sqrtf((float)r2)) / (float)W))
                          : 0.5 + 0.5 * tanh(2.0 * (R - sqrt(r2)) / W);
 }
@@ -409,7 +409,7 @@ __global__ void k_init_droplet(const uint8_t* __restrict__ cls, double* __restri
 {
     // the profile does not depend on the field: it is evaluated before the wait
     // for the droplet before this one
-    double v = 0.0;
+    double v = -INFINITY;
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     int y = ylo + blockIdx.y * blockDim.y + threadIdx.y;
     const bool in = i < xw && y < yhi;
@@ -418,7 +418,8 @@ __global__ void k_init_droplet(const uint8_t* __restrict__ cls, double* __restri
     const size_t k = (size_t)y * pitch + x;
     if (in && zeta_of(cls[k])) v = droplet_profile<F32>(x, y, nx, x0, y0, R, W, reach);
     step_wait();
-    if (in && (REPLACE || v > phi[k])) phi[k] = v;
+    if (in && REPLACE) phi[k] = v > 0.0 ? v : 0.0;   // the maximum with a cleared field
+    else if (in && v > phi[k]) phi[k] = v;
 }
 
 // The initial state in one pass: ghost values of phi0 (Sec. 2.2.2), mu of the
