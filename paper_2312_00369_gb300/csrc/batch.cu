@@ -58,10 +58,12 @@ struct pflbm_batch {
     std::vector<ClassLaunch> rest;
     uint4* d_items = nullptr;
     ResidentCut* d_cuts = nullptr;
-    void* d_words = nullptr;
-    size_t cap_items = 0, cap_cuts = 0, cap_words = 0;   // bytes
+    // exchange words and the lists' overflow, in buffers of their own: whatever
+    // members come and go, the words' memory holds zeros or words of earlier tags
+    // only (list entries there could be taken for a word that has arrived)
+    void *d_words = nullptr, *d_spill = nullptr;
+    size_t cap_items = 0, cap_cuts = 0, cap_words = 0, cap_spill = 0;   // bytes
     unsigned long long half_words = 0;     // exchange words of one buffer
-    size_t spill_at = 0;                   // byte offset of the lists' overflow in d_words
     unsigned res_tag = 0;
     // per-class launches run side by side: forked from the batch's stream to
     // these streams and joined back (in the captured graph as well)
@@ -308,14 +310,14 @@ int plan_waves(pflbm_batch_t* b, std::vector<int>* idx)
         b->half_words = std::max(b->half_words, at);
         b->waves.push_back(wv);
     }
-    b->spill_at = 2 * b->half_words * resident_word_bytes();
-    const size_t bytes = b->spill_at + (size_t)most * resident_spill(b->precision, cls) * 4;
+    const size_t bytes = 2 * b->half_words * resident_word_bytes();
     const bool fresh = bytes > b->cap_words;
     void *pi = b->d_items, *pc = b->d_cuts;
     int rc = grow(b, &pi, &b->cap_items, items.size() * sizeof(uint4));
     b->d_items = (uint4*)pi;
     if (!rc) rc = grow(b, &pc, &b->cap_cuts, cuts.size() * sizeof(ResidentCut));
     b->d_cuts = (ResidentCut*)pc;
+    if (!rc) rc = grow(b, &b->d_spill, &b->cap_spill, (size_t)most * resident_spill(b->precision, cls) * 4);
     if (!rc) rc = grow(b, &b->d_words, &b->cap_words, bytes);
     if (rc) {   // no memory for it: all members take single steps
         b->waves.clear();
@@ -584,7 +586,7 @@ int step_waves(pflbm_batch_t* b, int64_t n)
             const int c = (int)std::min<int64_t>(left, kResidentMaxSteps);
             cudaError_t e = cudaSuccess;
             if (b->res_tag > UINT_MAX - 2u * kResidentMaxSteps) {   // tags start again
-                e = cudaMemsetAsync(b->d_words, 0, b->spill_at, b->stream);
+                e = cudaMemsetAsync(b->d_words, 0, b->cap_words, b->stream);
                 b->res_tag = 0;
             }
             ResidentWave a{};
@@ -593,7 +595,7 @@ int step_waves(pflbm_batch_t* b, int64_t n)
             a.items = b->d_items + w.first;
             a.words = b->d_words;
             a.half = b->half_words;
-            a.spill = (uint32_t*)((char*)b->d_words + b->spill_at);
+            a.spill = (uint32_t*)b->d_spill;
             a.tag = b->res_tag;
             a.steps = c;
             a.n_items = w.count;
@@ -733,6 +735,7 @@ void pflbm_batch_destroy(pflbm_batch_t* b)
     bfree(b, b->d_items, b->cap_items);
     bfree(b, b->d_cuts, b->cap_cuts);
     bfree(b, b->d_words, b->cap_words);
+    bfree(b, b->d_spill, b->cap_spill);
     delete b;
 }
 
