@@ -317,6 +317,11 @@ void pflbm_batch_destroy(pflbm_batch_t* b);
  * build, 0 in the normal one; *violations: accesses refused so far on the
  * current device (0 in the normal build). Not in the paper: a test aid. */
 int pflbm_debug_bounds(int* enabled, unsigned* violations);
+/* Test aid, for one batch: *waves is the number of waves of members that a run
+ * of n steps would take resident (0: launches only); refuse_after >= 0: after
+ * that many more resident launches the next is taken as refused, as when fewer
+ * SMs are to be had than the device reports (< 0: none). */
+int pflbm_debug_batch(pflbm_batch_t* b, int64_t n, int refuse_after, int* waves);
 
 /* Text of the calling thread's last error ("" if none). */
 const char* pflbm_last_error(void);

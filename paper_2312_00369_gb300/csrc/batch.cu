@@ -53,8 +53,13 @@ struct pflbm_batch {
     // runs of many steps: members that fit the chip's shared memory are stepped
     // there (resident.cu), as many of them side by side as it holds (a wave),
     // wave by wave; the others as above (their own groups and graph)
-    struct Wave { int first, count; };     // its items
+    struct Wave {
+        int first, count;                  // its items
+        std::vector<int> members;
+    };
     std::vector<Wave> waves;
+    bool no_resident = false;              // a cooperative launch was refused: launches from then on
+    int refuse_after = -1;                 // test aid: resident launches until one is taken as refused
     std::vector<ClassLaunch> rest;
     uint4* d_items = nullptr;
     ResidentCut* d_cuts = nullptr;
@@ -245,7 +250,7 @@ int plan_waves(pflbm_batch_t* b, std::vector<int>* idx)
     int coop = 0, sms = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, b->device);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
-    if (!coop || cls < 0) return PFLBM_OK;
+    if (!coop || cls < 0 || b->no_resident) return PFLBM_OK;
     if (b->precision == PFLBM_FP32 && b->nodes > kResidentMaxNodes32) return PFLBM_OK;
     const int n = (int)b->hs.size();
     struct Member { int i, active; ResidentCut cut; unsigned long long words; };
@@ -294,12 +299,13 @@ int plan_waves(pflbm_batch_t* b, std::vector<int>* idx)
     int most = 0;
     b->half_words = 0;
     for (int w = 0; w < nw; ++w) {
-        pflbm_batch::Wave wv{(int)items.size(), 0};
+        pflbm_batch::Wave wv{(int)items.size(), 0, {}};
         unsigned long long at = 0;
         for (size_t k = 0; k < ms.size(); ++k) {
             if (wave[k] != w) continue;
             const Member& m = ms[k];
             cuts[m.i] = m.cut;
+            wv.members.push_back(m.i);
             for (int p = 0; p < m.cut.px * m.cut.py; ++p)
                 if (m.cut.active[p >> 5] >> (p & 31) & 1u)
                     items.push_back(make_uint4((unsigned)m.i, (unsigned)p, (unsigned)at, (unsigned)(at >> 32)));
@@ -308,7 +314,7 @@ int plan_waves(pflbm_batch_t* b, std::vector<int>* idx)
         wv.count = (int)items.size() - wv.first;
         most = std::max(most, wv.count);
         b->half_words = std::max(b->half_words, at);
-        b->waves.push_back(wv);
+        b->waves.push_back(std::move(wv));
     }
     const size_t bytes = 2 * b->half_words * resident_word_bytes();
     const bool fresh = bytes > b->cap_words;
@@ -577,16 +583,48 @@ bool capturing(cudaStream_t stream)
     return cudaStreamIsCapturing(stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
 }
 
+// A resident launch; cudaErrorCooperativeLaunchTooLarge and the like when fewer
+// SMs are to be had than the device reports.
+cudaError_t launch_wave(pflbm_batch_t* b, const ResidentWave& a, int cls)
+{
+    if (b->refuse_after >= 0 && b->refuse_after-- == 0) return cudaErrorCooperativeLaunchTooLarge;
+    return launch_resident_wave(b->precision, a, cls, b->stream);
+}
+
+// n steps of the members `idx` from parity `phase` on, one launch per size group
+// and step. Each member's copy named by its handle is that of the batch's phase.
+int step_members(pflbm_batch_t* b, const std::vector<int>& idx, int phase, int64_t n)
+{
+    std::vector<unsigned char> a0(b->args_bytes * b->hs.size()), a1(b->args_bytes * b->hs.size());
+    for (int i : idx) {
+        write_step_args(b->hs[i], b->phase, a0.data() + b->args_bytes * i);
+        write_step_args(b->hs[i], b->phase ^ 1, a1.data() + b->args_bytes * i);
+    }
+    const std::vector<pflbm_batch::ClassLaunch> classes = build_classes(b, idx, a0, a1);
+    for (int64_t left = n; left > 0;) {
+        const int c = (int)std::min<int64_t>(left, kResidentMaxSteps);
+        cudaError_t e = launch_steps(b, classes, phase, c);
+        if (e != cudaSuccess) return set_error(PFLBM_ECUDA, cudaGetErrorString(e));
+        phase ^= c & 1;
+        left -= c;
+    }
+    return PFLBM_OK;
+}
+
+// n steps of the waves' members. When a launch is refused, what is left of its
+// wave and the waves after it are taken by the size groups' launches, each from
+// the copy that it has come to, and so is everything from then on.
 int step_waves(pflbm_batch_t* b, int64_t n)
 {
     const int cls = resident_batch_class(b->precision);
     for (const pflbm_batch::Wave& w : b->waves) {
         int phase = b->phase;
-        for (int64_t left = n; left > 0;) {
+        int64_t left = n;
+        while (left > 0 && !b->no_resident) {
             const int c = (int)std::min<int64_t>(left, kResidentMaxSteps);
-            cudaError_t e = cudaSuccess;
             if (b->res_tag > UINT_MAX - 2u * kResidentMaxSteps) {   // tags start again
-                e = cudaMemsetAsync(b->d_words, 0, b->cap_words, b->stream);
+                cudaError_t e = cudaMemsetAsync(b->d_words, 0, b->cap_words, b->stream);
+                if (e != cudaSuccess) return set_error(PFLBM_ECUDA, cudaGetErrorString(e));
                 b->res_tag = 0;
             }
             ResidentWave a{};
@@ -599,14 +637,25 @@ int step_waves(pflbm_batch_t* b, int64_t n)
             a.tag = b->res_tag;
             a.steps = c;
             a.n_items = w.count;
-            if (e == cudaSuccess) e = launch_resident_wave(b->precision, a, cls, b->stream);
-            if (e != cudaSuccess) return set_error(PFLBM_ECUDA, cudaGetErrorString(e));
+            if (launch_wave(b, a, cls) != cudaSuccess) {
+                cudaGetLastError();
+                b->no_resident = true;
+                break;
+            }
             b->res_tag += (unsigned)c;
             phase ^= c & 1;
             left -= c;
         }
+        if (left > 0)
+            if (int rc = step_members(b, w.members, phase, left)) return rc;
     }
     return PFLBM_OK;
+}
+
+// Whether a run of n steps takes the waves.
+bool runs_resident(const pflbm_batch_t* b, int64_t n)
+{
+    return !b->waves.empty() && !b->no_resident && n >= kResidentMinSteps;
 }
 
 }  // namespace
@@ -683,7 +732,7 @@ int pflbm_batch_step(pflbm_batch_t* b, int64_t n)
     if (stale) {  // a member was stepped on its own: rewrite the descriptors
         if (int rc = upload(b)) return rc;
     }
-    if (!b->waves.empty() && n >= kResidentMinSteps && !capturing(b->stream)) {
+    if (runs_resident(b, n) && !capturing(b->stream)) {
         if (int rc = step_waves(b, n)) return rc;
         if (!b->rest.empty())
             if (int rc = step_launches(b, b->rest, &b->rest_graph, b->phase, n)) return rc;
@@ -713,6 +762,14 @@ int pflbm_batch_info(const pflbm_batch_t* b, int* n_work, int* grid, int64_t* no
     if (n_work) *n_work = b->n_work;
     if (grid) *grid = b->grid;
     if (nodes) *nodes = b->nodes;
+    return PFLBM_OK;
+}
+
+int pflbm_debug_batch(pflbm_batch_t* b, int64_t n, int refuse_after, int* waves)
+{
+    if (!b) return set_error(PFLBM_EINVAL, "batch: NULL batch");
+    b->refuse_after = refuse_after;
+    if (waves) *waves = runs_resident(b, n) ? (int)b->waves.size() : 0;
     return PFLBM_OK;
 }
 

@@ -58,3 +58,44 @@ def test_members_large_small_large(precision):
     b.close()
     for s in many + one:
         s.close()
+
+
+@pytest.mark.parametrize("refuse_after", [0, 1, 2, 3])
+@pytest.mark.parametrize("before", [0, 3])
+def test_refused_launch_falls_back(refuse_after, before):
+    """A refused cooperative launch: before any, after one wave's first launch of
+    1024 steps, between waves, in a later wave, from either phase. The batch takes
+    the launches for what is left and stays with them."""
+    from paper_2312_00369_gb300.pflbm import Batch, Solver
+    stream = torch.cuda.Stream()
+    sizes = [(192, 96), (192, 96), (320, 160), (256, 256), (100, 50), (300, 200), (256, 256), (256, 256), (256, 256)]
+    def make(kernel):
+        out = []
+        for i, (nx, ny) in enumerate(sizes):
+            s = Solver(dense(nx, ny, 3, 40), theta_deg=50.0 + 10 * i, precision="fp16", step_kernel=kernel, stream=stream,
+                       dgdt_mode=1)
+            s.init_droplet(0.4 * nx, 0.5 * ny, 0.3 * ny)
+            out.append(s)
+        return out
+    many, one = make("default"), make("global")
+    b = Batch(many)
+    n = 1029
+    b.step(before)
+    assert b.debug(n, refuse_after) >= 2
+    b.step(n)
+    assert b.debug(n) == 0
+    b.step(17)
+    b.set(many[:3])
+    b.step(20)
+    for s in one:
+        s.step(before + n + 17)
+    for s in one[:3]:
+        s.step(20)
+    for x, y, size in zip(many, one, sizes):
+        assert x.steps == y.steps
+        for p, q, what in zip(x.get() + (x.mass(),), y.get() + (y.mass(),), "phi u p mass".split()):
+            assert np.array_equal(p, q), (size, what)
+        x.check()
+    b.close()
+    for s in many + one:
+        s.close()
