@@ -103,9 +103,9 @@ typedef struct {
      * of a lattice that fits the chip's shared memory (up to about 270,000
      * fluid nodes in FP32, 310,000 in 16-bit storage, 75,000 in FP64) are
      * then taken many steps per launch, the lattice held there (they
-     * allocate exchange memory on first use, beyond
-     * pflbm_footprint_bytes; without it, and on a stream under capture,
-     * the steps run one launch each);
+     * allocate exchange memory on first use, which pflbm_footprint_bytes
+     * covers; without it, and on a stream under capture, the steps run one
+     * launch each);
      * 1: populations pulled from global memory, 32 x 8 tiles; 2:
      * populations staged in shared memory by TMA, 32 x 8 tiles; 3: staged,
      * 64 x 4 tiles; 4: global loads, two x-adjacent nodes per thread in
@@ -233,7 +233,12 @@ int pflbm_status(const pflbm_t* h);
 /* Steps taken since the last initialisation. */
 int64_t pflbm_steps(const pflbm_t* h);
 
-/* Device bytes a handle of this size and precision allocates. */
+/* Device bytes a handle of this size and precision allocates at most, beside an
+ * angle field (4 bytes per padded node) and the scratch of the float
+ * read-back (16 bytes per node). Part of it is taken on first use: the
+ * scratch of the FP64 read-back, and the exchange memory of runs of many
+ * steps (lattices of up to about 300,000 fluid nodes; its size depends on the
+ * mask, and the largest is counted). */
 size_t pflbm_footprint_bytes(int nx, int ny, int precision);
 
 /* Checkpoint: *len in: capacity of buf, out: bytes needed/written. buf may be
@@ -290,7 +295,8 @@ typedef struct {
  * default kernel, no size classes. */
 void pflbm_schedule_default(pflbm_schedule_t* s);
 /* Build a batch over hs[0..count-1] (schedule NULL: defaults). Allocates the
- * device work list and descriptors with cudaMalloc. EINVAL if the handles
+ * device work list and descriptors with cudaMalloc, and for resident runs up to
+ * 50 MB of exchange memory, whatever its members. EINVAL if the handles
  * differ in precision, device or stream, or repeat. Members may be destroyed
  * while the batch lives, as long as pflbm_batch_set drops them before the
  * next pflbm_batch_step. */

@@ -306,9 +306,10 @@ int plan_waves(pflbm_batch_t* b, std::vector<int>* idx)
             const Member& m = ms[k];
             cuts[m.i] = m.cut;
             wv.members.push_back(m.i);
+            unsigned rank = 0;
             for (int p = 0; p < m.cut.px * m.cut.py; ++p)
                 if (m.cut.active[p >> 5] >> (p & 31) & 1u)
-                    items.push_back(make_uint4((unsigned)m.i, (unsigned)p, (unsigned)at, (unsigned)(at >> 32)));
+                    items.push_back(make_uint4((unsigned)m.i, rank++ << 16 | (unsigned)p, (unsigned)at, (unsigned)(at >> 32)));
             at += m.words;
         }
         wv.count = (int)items.size() - wv.first;
@@ -323,7 +324,7 @@ int plan_waves(pflbm_batch_t* b, std::vector<int>* idx)
     b->d_items = (uint4*)pi;
     if (!rc) rc = grow(b, &pc, &b->cap_cuts, cuts.size() * sizeof(ResidentCut));
     b->d_cuts = (ResidentCut*)pc;
-    if (!rc) rc = grow(b, &b->d_spill, &b->cap_spill, (size_t)most * resident_spill(b->precision, cls) * 4);
+    if (!rc) rc = grow(b, &b->d_spill, &b->cap_spill, (size_t)most * resident_spill(b->precision, cls).words() * 4);
     if (!rc) rc = grow(b, &b->d_words, &b->cap_words, bytes);
     if (rc) {   // no memory for it: all members take single steps
         b->waves.clear();

@@ -251,6 +251,12 @@ constexpr int64_t kResidentMinSteps = 16;
 constexpr int kResidentMaxSteps = 1024;          // steps of one launch: a few milliseconds
 constexpr long long kResidentMapNodes = 1 << 20; // larger lattices never fit
 
+// What a handle may allocate for them, whatever its mask.
+size_t resident_allowance(int nx, int ny, int precision)
+{
+    return (long long)nx * ny <= kResidentMapNodes ? resident_bytes_at_most(nx, ny, precision) : 0;
+}
+
 bool capturing(cudaStream_t stream)
 {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
@@ -269,13 +275,23 @@ bool resident_ready(pflbm_t* h)
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     if (!coop || !plan_resident(h->nx, h->ny, h->precision, h->map, sms, -1, &h->res)) return false;
+    // what the lists need past shared memory (nothing, but for dense obstacles):
+    // dstatus[2..3] and hstatus[2..3] are for this alone
+    h->res_tag = 0;
+    if (cudaMemsetAsync(h->dstatus + 2, 0, 2 * sizeof(int), h->stream) != cudaSuccess ||
+        launch_resident(h, h->res, 0, h->dstatus + 2) != cudaSuccess ||
+        cudaMemcpyAsync(h->hstatus + 2, h->dstatus + 2, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
+        cudaStreamSynchronize(h->stream) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (!add_spill(&h->res, h->hstatus + 2)) return false;
     void* p = nullptr;
     if (h->alloc_fn) p = h->alloc_fn(h->res.bytes, h->alloc_ctx);
     else if (cudaMalloc(&p, h->res.bytes) != cudaSuccess) { cudaGetLastError(); p = nullptr; }
     if (!p) return false;                        // single steps need no more memory
     h->bytes_allocated += h->res.bytes;
     h->res_words = p;
-    h->res_tag = 0;
     if (cudaMemsetAsync(p, 0, h->res.bytes, h->stream) != cudaSuccess) { cudaGetLastError(); return false; }
     h->res_state = 1;
     return true;
@@ -360,10 +376,9 @@ size_t pflbm_footprint_bytes(int nx, int ny, int precision)
 {
     if (nx < 1 || ny < 1) return 0;
     Sizes s = sizes_of(nx, ny, precision);
-    // (of the 26 bytes per node beside the state, 8 are an allowance for the
-    // exchange memory of resident runs, allocated on first use)
-    return 2 * s.pop + s.sprev + s.wet + s.N * (1 + 1 + 8 + 8 + 8) + s.red + s.pts + s.tiles + 16 +
-           (size_t)nx * ny * 4 * sizeof(double) +
+    // cls, solid, av, phi0; FP64 read-back; exchange memory of resident runs
+    return 2 * s.pop + s.sprev + s.wet + s.N * (1 + 1 + 8 + 8) + s.red + s.pts + s.tiles + 16 +
+           (size_t)nx * ny * 4 * sizeof(double) + resident_allowance(nx, ny, precision) +
            (precision != PFLBM_FP64 ? tma_sets_bytes() + staged_flags_bytes(nx, ny) + node_words_bytes(nx, ny) +
                                           tile2_flags_bytes(nx, ny)
                                     : 0);

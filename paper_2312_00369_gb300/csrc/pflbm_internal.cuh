@@ -166,13 +166,21 @@ constexpr int kMaxPatches = 1024;
 struct ResidentCut {
     int px, py;
     int units, rows;                    // columns / nodes per lane (rounded up), ny - 2
-    int max_slots;                      // exchange words per type and patch
+    int w, h;                           // the largest patch
     uint32_t active[kMaxPatches / 32];
+    uint16_t before[kMaxPatches / 32];  // active patches below each word of the set
+};
+// Room for entries of a patch's lists in global memory (poll, its cells, publish:
+// the same each; bounce-back copies).
+struct ResidentSpill {
+    int list, copies;
+    __host__ __device__ constexpr int words() const { return 3 * list + copies; }   // 32-bit words
 };
 struct ResidentPlan {
     ResidentCut cut{};
     int cls = 0, nt = 0, n_active = 0;  // patch class, threads per CTA, CTAs
     unsigned long long words = 0;       // exchange words (both buffers)
+    ResidentSpill room{0, 0};
     size_t bytes = 0;                   // the words and the lists' overflow
 };
 // 8 x 8 blocks with a fluid node, as a summed-area table.
@@ -185,7 +193,7 @@ struct SolidMap {
 struct ResidentWave {
     const void* args;                   // step descriptors (device)
     const ResidentCut* cuts;
-    const uint4* items;                 // member, patch, first word (64 bits)
+    const uint4* items;                 // member, patch and its rank, first word (64 bits)
     void* words;
     unsigned long long half;
     uint32_t* spill;
@@ -288,9 +296,15 @@ int resident_batch_class(int precision);              // patch class of batches;
 // words (one buffer).
 bool cut_resident(int nx, int ny, int precision, const SolidMap& map, int cls, double split, ResidentCut* cut,
                   int* n_active, unsigned long long* half_words);
-int resident_spill(int precision, int cls);           // 32-bit words of list overflow per CTA
+ResidentSpill resident_spill(int precision, int cls);   // room per CTA of a batch
+// Takes the overflow that a launch of 0 steps found into the plan; false: more
+// than a handle's footprint allows for.
+bool add_spill(ResidentPlan* plan, const int need[2]);
+// Upper bound of ResidentPlan::bytes for any mask of this size.
+size_t resident_bytes_at_most(int nx, int ny, int precision);
 cudaError_t launch_resident_wave(int precision, const ResidentWave& w, int cls, cudaStream_t stream);
-cudaError_t launch_resident(pflbm_t* h, const ResidentPlan& plan, int steps);
+// (steps = 0: only the largest overflow of a list and of the copies, into need[0..1])
+cudaError_t launch_resident(pflbm_t* h, const ResidentPlan& plan, int steps, int* need = nullptr);
 unsigned bounds_violations_resident();
 // step2.cu: two x-adjacent nodes per thread in packed FP32x2 (FP32, 16-bit)
 cudaError_t launch_step2(pflbm_t* h);

@@ -61,7 +61,7 @@ namespace {
 // us and more), so some seconds; in a healthy run a word is there within a step.
 constexpr int kSpinLimit = 1 << 22;
 constexpr int kHaloX = 4, kHaloY = 3;   // three nodes are read; four in x keeps pairs aligned
-constexpr int kMaxResident = 256;       // CTAs of a one-lattice launch at most
+constexpr int kMaxResident = 152;       // CTAs of a one-lattice launch at most (one per SM)
 
 // A word of the exchange: three 32-bit payloads and the step tag, one 128-bit
 // access of memory.
@@ -122,25 +122,51 @@ __host__ __device__ __forceinline__ Rect patch_rect(const ResidentCut& c, int id
     return r;
 }
 
-// Place of a border node's word within its plane: the three bottom rows, the
-// three top rows, then the three columns at each side.
-__device__ __forceinline__ int slot_of(const Rect& r, int lx, int ly)
+// Place of the word of type t of a border node among its patch's words. A type
+// that crosses horizontal borders takes rows of nodes, one that crosses
+// vertical ones columns: of f the outermost at each side (what a pull reaches),
+// of g the three outermost (a pull on the ring of one, or of two next to a
+// ghost), so 24 (w + h) words in all. Words of nodes side by side lie side by
+// side, three columns' as rows of three (column after column a step of 512 x 512
+// FP32 took 5.99 us instead of 5.79).
+// ROOMY (batches, whose words are one buffer however many the members): the place
+// among the type's, each of which takes all 6 (w + h) border nodes, rows first.
+// With the compact places a step of 256 uneven lattices in BF16 took 179 us
+// instead of 175.
+template <bool ROOMY>
+__device__ __forceinline__ int slot_of(const ResidentCut& c, const Rect& r, int t, int lx, int ly)
 {
-    if (ly < 3) return ly * r.w + lx;
-    if (ly >= r.h - 3) return (3 + ly - (r.h - 3)) * r.w + lx;
-    if (lx < 3) return 6 * r.w + ly * 6 + lx;
-    return 6 * r.w + ly * 6 + 3 + lx - (r.w - 3);
+    const int row = ly < 3 ? ly : ly - r.h + 6, col = lx < 3 ? lx : lx - r.w + 6;
+    if (ROOMY) return ly < 3 || ly >= r.h - 3 ? row * r.w + lx : 6 * r.w + ly * 6 + col;
+    const int tt = t % 6, g = 6 * (c.w + c.h);
+    if (tt < 3) return t < 6 ? (2 * tt + (ly != 0)) * c.w + lx : g + (6 * tt + row) * c.w + lx;
+    if (t < 6) return 6 * c.w + (2 * (tt - 3) + (lx != 0)) * c.h + ly;
+    return g + 18 * c.w + (6 * (tt - 3) + (lx < 3 ? 0 : 3)) * c.h + 3 * ly + col % 3;
 }
 
-// Words of a patch in one buffer: its types' slots, then the heartbeat in a line
-// of its own.
+// Words of a patch in one buffer: its types' places, then the heartbeat in a line
+// of its own. Only active patches have words, in their order.
 constexpr int kHeartbeat = 8;
-__host__ __device__ __forceinline__ int patch_words(const ResidentCut& c) { return (kTypes * c.max_slots + 7) / 8 * 8 + kHeartbeat; }
+template <bool ROOMY> __host__ __device__ __forceinline__ int patch_words(int w, int h) { return (ROOMY ? 72 : 24) * (w + h) + kHeartbeat; }
+// (places of a ROOMY patch count from the type's first word)
+template <bool ROOMY> __device__ __forceinline__ int type_words(const ResidentCut& c) { return ROOMY ? 6 * (c.w + c.h) : 0; }
+// An entry of the publish list: type, place, cell. (Two orders of the bits: the
+// other order costs 0.5 to 1.5 % of a step in each case.)
+template <bool ROOMY> __device__ __forceinline__ uint32_t pub_entry(int t, int slot, int c)
+{
+    return ROOMY ? (uint32_t)t << 28 | (uint32_t)slot << 13 | (uint32_t)c : (uint32_t)slot << 17 | (uint32_t)t << 13 | (uint32_t)c;
+}
+template <bool ROOMY> __device__ __forceinline__ unsigned pub_type(uint32_t u) { return ROOMY ? u >> 28 : (u >> 13) & 0xfu; }
+template <bool ROOMY> __device__ __forceinline__ unsigned pub_slot(uint32_t u) { return ROOMY ? (u >> 13) & 0x7fffu : u >> 17; }
+template <bool ROOMY> __device__ __forceinline__ int first_word(const ResidentCut& c, int id)
+{
+    return (c.before[id >> 5] + __popc(c.active[id >> 5] & ((1u << (id & 31)) - 1u))) * patch_words<ROOMY>(c.w, c.h);
+}
 
 // Shared memory of a patch of at most WM x HM nodes: byte offsets of the
 // arrays. Row and plane strides are constants, so a pull's offset is an
 // immediate of its load.
-constexpr int kMaxList(int w, int h) { return 8 * 2 * (w + h) + 512; }
+constexpr int kMaxList(int w, int h) { return 8 * 2 * (w + h) + 512; }   // entries of an exchange list at most
 constexpr int align16(int b) { return (b + 15) & ~15; }
 template <int PREC, int WM, int HM>
 struct Lay {
@@ -162,29 +188,33 @@ struct Lay {
     // bounce-back copies: up to 3 unknown links per node of a wall are usual;
     // more than the list holds wait in global memory
     static constexpr int COPIES = 6 * (WM + HM) + 64, MAXCOPY = 8 * (WM + 4) * (HM + 4);
+    // whole lists, which no mask can exceed
+    static constexpr ResidentSpill kMost{MAXLIST, MAXCOPY};
     static constexpr int kCopy = kGhost + align16((WM + 2) * (HM + 2) * 4);
     static constexpr int kPoll = kCopy + align16(COPIES * 4);
     static constexpr int kPollC = kPoll + align16(CAP * 4);
     static constexpr int kPub = kPollC + align16(CAP * 2);
-    static constexpr int SPILL = 3 * MAXLIST + MAXCOPY;
     static constexpr int kBytes = kPub + align16(CAP * 4);
     static_assert(9 * CELLS <= 32768 && CELLS <= 8192, "packed offsets of the lists");
     static_assert(kBytes <= 227 * 1024 - 1024, "shared memory of one CTA");
 };
 
 // One lattice: its descriptor and cut are launch parameters. A batch: CTA b
-// runs patch item[b].y of member item[b].x, whose words start at item[b].zw.
+// runs patch item[b].y (its place among the active ones in the upper half) of
+// member item[b].x, whose words start at item[b].zw.
 template <int PREC, bool BATCH> struct ResArgs;
 struct ResCommon {
     Word* ll;                        // two buffers of ll_half words
     unsigned long long ll_half;
-    uint32_t* spill;                 // list entries past what shared memory holds: SPILL per CTA
+    uint32_t* spill;                 // list entries past what shared memory holds
     unsigned tag;                    // words of step s carry tag + s
     int steps;
 };
 template <int PREC> struct ResArgs<PREC, false> : ResCommon {
     StepArgs<PREC> a;
     ResidentCut cut;
+    ResidentSpill room;              // of each CTA in spill (batches: Lay::kMost)
+    int* need;                       // steps = 0: only the largest overflow of a list and of the copies
     uint16_t item[kMaxResident];     // patch of each CTA
 };
 template <int PREC> struct ResArgs<PREC, true> : ResCommon {
@@ -367,7 +397,7 @@ __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ R
     const StepArgs<PREC>* ap;
     const ResidentCut* cp;
     Word* ll = q.ll;
-    int id;
+    int id, rank = 0;                             // patch; its place among the member's active ones
     if constexpr (BATCH) {
         // the member's descriptor and cut, read field by field where used
         const uint4 it = q.item[blockIdx.x];
@@ -379,7 +409,8 @@ __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ R
             reinterpret_cast<int*>(s_arg)[i] = i < NA ? sa[i] : sc[i - NA];
         ap = reinterpret_cast<const StepArgs<PREC>*>(s_arg);
         cp = reinterpret_cast<const ResidentCut*>(s_arg + sizeof(StepArgs<PREC>));
-        id = (int)it.y;
+        id = (int)(it.y & 0xffffu);
+        rank = (int)(it.y >> 16);
         ll += (unsigned long long)it.w << 32 | it.z;
         __syncthreads();
     } else {
@@ -409,8 +440,19 @@ __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ R
     uint16_t* sPollC = reinterpret_cast<uint16_t*>(sm + L::kPollC);
     uint32_t* sPub = reinterpret_cast<uint32_t*>(sm + L::kPub);
 
-    uint32_t* gPoll = q.spill + (size_t)blockIdx.x * L::SPILL;
-    uint32_t *gPollC = gPoll + L::MAXLIST, *gPub = gPollC + L::MAXLIST, *gCopy = gPub + L::MAXLIST;
+    // entry `at` of the lists (0: poll, 1: its cell, 2: publish) and of the copies
+    // past shared memory, in the CTA's part of the overflow. A batch's has room
+    // for whole lists, list by list.
+    int room_list = L::MAXLIST, room_copy = L::MAXCOPY;
+    uint32_t* gList = q.spill + (size_t)blockIdx.x * L::kMost.words();
+    uint32_t* gCopy = gList + 3 * L::MAXLIST;
+    if constexpr (!BATCH) {
+        room_list = L::CAP + q.room.list;
+        room_copy = L::COPIES + q.room.copies;
+        gList = q.spill + (size_t)blockIdx.x * q.room.words() - 3 * L::CAP;
+        gCopy = gList + 3 * room_list - L::COPIES;
+    }
+    auto over = [&](int list, int at) { return gList + (BATCH ? list * L::MAXLIST + at : 3 * at + list); };
 
     // ---- set-up: the state, the node words, the lists ----
     if (tid < 6) s_n[tid] = 0;
@@ -430,6 +472,8 @@ __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ R
         const bool in = gy >= 0 && gy < ny;
         const int k = in ? gy * pitch + wrapn(r.x0 + lx, nx) : 0;
         sW[c] = in ? PFLBM_LD(a.cls, k, plane) : (uint8_t)CLS_OUT;
+        mask[c] = 0;
+        if (!BATCH && q.steps == 0) continue;
         sG0[c] = in ? PFLBM_LD(a.in.g0, k, plane) : G0T(0);
 #pragma unroll
         for (int p = 0; p < 17; ++p) {
@@ -438,7 +482,6 @@ __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ R
             else v = PFLBM_LD(a.in.g, (p - 8) * plane + (in ? k : 0), 9LL * plane);
             sS[p * cells + c] = v;
         }
-        mask[c] = 0;
         if (lx >= 0 && lx < w2 && ly >= 0 && ly < r.h) {
             const int o = ly * WM + lx;
             const bool own = lx < r.w;
@@ -493,7 +536,7 @@ __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ R
                 const uint32_t dst = (uint32_t)(i * cells + c - (cy(i) * rs + cx(i)));
                 const uint32_t from = (uint32_t)(o * cells + c + dy * rs + dx);
                 const int at = atomicAdd(&s_n[4], 1);
-                if (at < L::MAXCOPY)
+                if (at < room_copy)
                     (at < L::COPIES ? sCopy + at : gCopy + at)[0] = (own ? 1u << 31 : 0u) | dst << 16 | from;
             }
         };
@@ -519,24 +562,24 @@ __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ R
                 int at = 0;
                 if ((tid & 31) == 0) at = atomicAdd(&s_n[side], __popc(m));
                 at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << (tid & 31)) - 1u));
-                if (!on || at >= L::MAXLIST) continue;
+                if (!on || at >= room_list) continue;
                 if (side == 1) {
-                    (at < L::CAP ? sPub + at : gPub + at)[0] =
-                        (uint32_t)p << 27 | (uint32_t)slot_of(r, lx, ly) << 13 | (uint32_t)c;
+                    (at < L::CAP ? sPub + at : over(2, at))[0] =
+                        pub_entry<BATCH>(p, slot_of<BATCH>(cut, r, p, lx, ly), c);
                 } else {
                     const int gx = wrapn(r.x0 + lx, nx), gy = r.y0 + ly;
                     const int i = ((gx / N + 1) * cut.px - 1) / cut.units, j = (gy * cut.py - 1) / cut.rows;
                     const int from = j * cut.px + i;
                     const Rect o = patch_rect<N>(cut, from, nx);
-                    const uint32_t u = (uint32_t)p << 28 | (uint32_t)(from * patch_words(cut) + p * cut.max_slots +
-                                                                      slot_of(o, gx - o.x0, gy - o.y0));
+                    const uint32_t u = (uint32_t)p << 28 | (uint32_t)(first_word<BATCH>(cut, from) + p * type_words<BATCH>(cut) +
+                                                                      slot_of<BATCH>(cut, o, p, gx - o.x0, gy - o.y0));
                     atomicOr(&s_seen[from >> 5], 1u << (from & 31));
                     if (at < L::CAP) {
                         sPoll[at] = u;
                         sPollC[at] = (uint16_t)c;
                     } else {
-                        gPoll[at] = u;
-                        gPollC[at] = (uint32_t)c;
+                        *over(0, at) = u;
+                        *over(1, at) = (uint32_t)c;
                     }
                 }
             }
@@ -554,19 +597,28 @@ __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ R
         if (s_seen[of >> 5] >> (of & 31) & 1u) continue;
         if (atomicOr(&s_seen[of >> 5], 1u << (of & 31)) >> (of & 31) & 1u) continue;
         const int at = atomicAdd(&s_n[0], 1);
-        const uint32_t u = (uint32_t)((of + 1) * patch_words(cut) - kHeartbeat);
+        const uint32_t u = (uint32_t)(first_word<BATCH>(cut, of) + patch_words<BATCH>(cut.w, cut.h) - kHeartbeat);
         if (at < L::CAP) {
             sPoll[at] = u;
             sPollC[at] = (uint16_t)(cells - 1);
-        } else if (at < L::MAXLIST) {
-            gPoll[at] = u;
-            gPollC[at] = (uint32_t)(cells - 1);
+        } else if (at < room_list) {
+            *over(0, at) = u;
+            *over(1, at) = (uint32_t)(cells - 1);
         }
     }
     __syncthreads();
     for (int c = tid; c < area; c += NT) sPhi[c] = R(0);
     const int n_poll = s_n[0], n_pub = s_n[1], n_ring = s_n[2], n_ghost = s_n[3], n_copy = s_n[4];
-    if (n_poll > L::MAXLIST || n_pub > L::MAXLIST || n_copy > L::MAXCOPY) {   // cannot happen (see Lay); nothing was written past the lists
+    if constexpr (!BATCH) {
+        if (q.steps == 0) {
+            if (tid == 0) {
+                atomicMax(&q.need[0], (n_poll > n_pub ? n_poll : n_pub) - L::CAP);
+                atomicMax(&q.need[1], n_copy - L::COPIES);
+            }
+            return;
+        }
+    }
+    if (n_poll > room_list || n_pub > room_list || n_copy > room_copy) {   // cannot happen (the room was worked out); nothing was written past the lists
         if (tid == 0) atomicOr(a.status, 4);
         return;
     }
@@ -732,13 +784,14 @@ __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ R
         constexpr int NS = (L::kPhi - L::kS) / (int)sizeof(S), NW = (L::kPhi - L::kS) / 4;   // elements of sS and sG0
         Word* buf = ll + (s & 1) * q.ll_half;
         {
-            Word* to = buf + (unsigned long long)id * patch_words(cut) * WPT;
-            if (tid < WPT) st_word(to + (patch_words(cut) - kHeartbeat) * WPT + tid, 0u, 0u, 0u, tag);
+            const int words = patch_words<BATCH>(cut.w, cut.h);
+            Word* to = buf + (unsigned long long)((BATCH ? rank : (int)blockIdx.x) * words) * WPT;
+            if (tid < WPT) st_word(to + (words - kHeartbeat) * WPT + tid, 0u, 0u, 0u, tag);
             for (int e = tid; e < n_pub; e += NT) {
-                const uint32_t u = e < L::CAP ? sPub[e] : gPub[e];
+                const uint32_t u = e < L::CAP ? sPub[e] : *over(2, e);
                 const int c = (int)(u & 0x1fffu);
-                Word* d = to + ((u >> 27) * cut.max_slots + ((u >> 13) & 0x3fffu)) * WPT;
-                const int4 off = s_off[u >> 27];
+                Word* d = to + (pub_type<BATCH>(u) * type_words<BATCH>(cut) + pub_slot<BATCH>(u)) * WPT;
+                const int4 off = s_off[pub_type<BATCH>(u)];
                 if constexpr (PREC == PFLBM_FP64) {
                     const double v0 = PFLBM_LD(sS, c + off.x, NS), v1 = PFLBM_LD(sS, c + off.y, NS),
                                  v2 = PFLBM_LD(sS, c + off.z, NS);
@@ -767,8 +820,8 @@ __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ R
             for (int u = 0; u < U; ++u) {
                 const int e = e0 + u * NT;
                 have[u] = e >= n_poll;
-                const uint32_t ent = have[u] ? 0u : e < L::CAP ? sPoll[e] : gPoll[e];
-                const int c = have[u] ? 0 : e < L::CAP ? (int)sPollC[e] : (int)gPollC[e];
+                const uint32_t ent = have[u] ? 0u : e < L::CAP ? sPoll[e] : *over(0, e);
+                const int c = have[u] ? 0 : e < L::CAP ? (int)sPollC[e] : (int)*over(1, e);
                 src[u] = buf + (ent & 0xfffffffu) * WPT;
                 off[u] = s_off[ent >> 28];
                 off[u].x += c;
@@ -858,19 +911,7 @@ constexpr Class class_of(int precision, int k)
 }
 constexpr int classes(int precision) { return precision == PFLBM_FP64 ? 2 : kClassCount; }
 
-template <int PREC, int K> constexpr int spill_k() { return Lay<PREC, class_of(PREC, K).wm, class_of(PREC, K).hm>::SPILL; }
-template <int PREC> int spill_prec(int k)
-{
-    if (k == 0) return spill_k<PREC, 0>();
-    if (k == 1) return spill_k<PREC, 1>();
-    if constexpr (PREC != PFLBM_FP64) return spill_k<PREC, 2>();
-    return 0;
-}
-// the layouts of the two 16-bit formats are the same
-int spill_of(int precision, int k)
-{
-    return precision == PFLBM_FP64 ? spill_prec<PFLBM_FP64>(k) : precision == PFLBM_FP32 ? spill_prec<PFLBM_FP32>(k) : spill_prec<PFLBM_BF16>(k);
-}
+template <int PREC, int K> constexpr ResidentSpill spill_k() { return Lay<PREC, class_of(PREC, K).wm, class_of(PREC, K).hm>::kMost; }
 
 template <int PREC, int VV, int K, bool BATCH>
 cudaError_t launch_k(const ResArgs<PREC, BATCH>& q, int n_items, int nt, cudaStream_t stream)
@@ -881,11 +922,12 @@ cudaError_t launch_k(const ResArgs<PREC, BATCH>& q, int n_items, int nt, cudaStr
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     void* args[] = {(void*)&q};
+    if (q.steps == 0) return cudaLaunchKernel((const void*)k, dim3(n_items), dim3(nt), args, smem, stream);   // no exchange
     return cudaLaunchCooperativeKernel((const void*)k, dim3(n_items), dim3(nt), args, smem, stream);
 }
 
 template <int PREC>
-cudaError_t launch_prec(pflbm_t* h, const ResidentPlan& pl, int steps)
+cudaError_t launch_prec(pflbm_t* h, const ResidentPlan& pl, int steps, int* need)
 {
     ResArgs<PREC, false> q;
     write_step_args(h, 0, &q.a);
@@ -893,6 +935,8 @@ cudaError_t launch_prec(pflbm_t* h, const ResidentPlan& pl, int steps)
     q.ll = (Word*)h->res_words;
     q.ll_half = pl.words / 2;
     q.spill = (uint32_t*)(q.ll + pl.words);
+    q.room = pl.room;
+    q.need = need;
     q.tag = h->res_tag;
     q.steps = steps;
     int n = 0;
@@ -961,6 +1005,16 @@ void SolidMap::build(const uint8_t* solid, int nx, int ny)
                                              sum[(size_t)(y - 1) * (bw + 1) + x - 1];
 }
 
+// active patches below each word of the set
+void count_before(ResidentCut* c)
+{
+    int n = 0;
+    for (int i = 0; i < kMaxPatches / 32; ++i) {
+        c->before[i] = (uint16_t)n;
+        n += __builtin_popcount(c->active[i]);
+    }
+}
+
 constexpr int kPlanTests = 30000;
 
 // The cut with the smallest estimated step: the collision and pulls of the
@@ -1005,7 +1059,8 @@ bool plan_resident(int nx, int ny, int precision, const SolidMap& map, int max_c
                 cut.py = py;
                 cut.units = units;
                 cut.rows = rows;
-                cut.max_slots = 6 * (w2 + h);
+                cut.w = w2;
+                cut.h = h;
                 int n = 0;
                 for (int i = 0; i < px * py && n <= cap; ++i, ++tests) {
                     const Rect r = unit == 1 ? patch_rect<1>(cut, i, nx) : patch_rect<2>(cut, i, nx);
@@ -1018,14 +1073,16 @@ bool plan_resident(int nx, int ny, int precision, const SolidMap& map, int max_c
                 if (n == 0) break;
                 best = cost;
                 found = true;
+                count_before(&cut);
                 out->cut = cut;
                 out->cls = k;
                 out->n_active = n;
                 const int per = ((lanes + c.p - 1) / c.p + 31) / 32 * 32;
                 // the exchange and the ring want threads too
                 out->nt = per < 256 ? 256 : per;
-                out->words = 2ull * px * py * patch_words(cut) * (precision == PFLBM_FP64 ? 2 : 1);
-                out->bytes = out->words * sizeof(Word) + (size_t)n * spill_of(precision, k) * 4;
+                out->words = 2ull * n * patch_words<false>(w2, h) * (precision == PFLBM_FP64 ? 2 : 1);
+                out->room = {0, 0};
+                out->bytes = out->words * sizeof(Word);
                 break;
             }
         }
@@ -1049,27 +1106,69 @@ bool cut_resident(int nx, int ny, int precision, const SolidMap& map, int cls, d
     if ((long long)cut->px * cut->py > kMaxPatches) return false;
     cut->units = units;
     cut->rows = rows;
-    cut->max_slots = 6 * ((units + cut->px - 1) / cut->px * 2 + (rows + cut->py - 1) / cut->py);
+    cut->w = (units + cut->px - 1) / cut->px * 2;
+    cut->h = (rows + cut->py - 1) / cut->py;
     int n = 0;
     for (int i = 0; i < cut->px * cut->py; ++i)
         if (patch_active(map, patch_rect<2>(*cut, i, nx), nx)) {
             cut->active[i >> 5] |= 1u << (i & 31);
             ++n;
         }
+    count_before(cut);
     *n_active = n;
-    *half_words = (unsigned long long)cut->px * cut->py * patch_words(*cut);
+    *half_words = (unsigned long long)n * patch_words<true>(cut->w, cut->h);
     return true;
 }
-int resident_spill(int precision, int cls) { return spill_of(precision, cls); }
+// (the layouts of the two 16-bit formats are the same)
+ResidentSpill resident_spill(int precision, int cls)
+{
+    if (precision == PFLBM_FP64) return cls == 0 ? spill_k<PFLBM_FP64, 0>() : spill_k<PFLBM_FP64, 1>();
+    if (precision == PFLBM_FP32)
+        return cls == 0 ? spill_k<PFLBM_FP32, 0>() : cls == 1 ? spill_k<PFLBM_FP32, 1>() : spill_k<PFLBM_FP32, 2>();
+    return cls == 0 ? spill_k<PFLBM_BF16, 0>() : cls == 1 ? spill_k<PFLBM_BF16, 1>() : spill_k<PFLBM_BF16, 2>();
+}
 
-cudaError_t launch_resident(pflbm_t* h, const ResidentPlan& pl, int steps)
+// The overflow that a handle's footprint allows for: 32-bit words per patch, an
+// eighth of its exchange words' memory. Dense obstacles need it: 5 x 5 solid
+// blocks every 8 nodes take about 900 of a 64 x 32 patch's 2304.
+static int spill_allowed(int w, int h) { return 24 * (w + h); }
+
+bool add_spill(ResidentPlan* pl, const int need[2])
+{
+    pl->room = {need[0] > 0 ? need[0] : 0, need[1] > 0 ? need[1] : 0};
+    if (pl->room.words() > spill_allowed(pl->cut.w, pl->cut.h)) return false;
+    pl->bytes = pl->words * sizeof(Word) + (size_t)pl->n_active * pl->room.words() * 4;
+    return true;
+}
+
+// The largest over all cuts that plan_resident may come to, whatever the mask.
+size_t resident_bytes_at_most(int nx, int ny, int precision)
+{
+    const int unit = precision == PFLBM_FP64 ? 1 : 2, units = (nx + unit - 1) / unit, rows = ny - 2;
+    const Class big = class_of(precision, classes(precision) - 1);
+    size_t most = 0;
+    for (int px = 1; px <= units && px <= kMaxPatches; ++px) {
+        const int w2 = (units + px - 1) / px * unit;
+        if (w2 > big.wm || (px > 1 && w2 / unit < 4)) continue;
+        for (int py = 1; py <= rows && py <= kMaxPatches / px; ++py) {
+            const int h = (rows + py - 1) / py, n = px * py < kMaxResident ? px * py : kMaxResident;
+            if (h > big.hm) continue;
+            const size_t bytes = n * (2 * patch_words<false>(w2, h) * (precision == PFLBM_FP64 ? 2 : 1) * sizeof(Word) +
+                                      spill_allowed(w2, h) * sizeof(uint32_t));
+            if (bytes > most) most = bytes;
+        }
+    }
+    return most;
+}
+
+cudaError_t launch_resident(pflbm_t* h, const ResidentPlan& pl, int steps, int* need)
 {
     cudaError_t e;
     switch (h->precision) {
-        case PFLBM_FP64: e = launch_prec<PFLBM_FP64>(h, pl, steps); break;
-        case PFLBM_FP32: e = launch_prec<PFLBM_FP32>(h, pl, steps); break;
-        case PFLBM_BF16: e = launch_prec<PFLBM_BF16>(h, pl, steps); break;
-        default: e = launch_prec<PFLBM_FP16>(h, pl, steps); break;
+        case PFLBM_FP64: e = launch_prec<PFLBM_FP64>(h, pl, steps, need); break;
+        case PFLBM_FP32: e = launch_prec<PFLBM_FP32>(h, pl, steps, need); break;
+        case PFLBM_BF16: e = launch_prec<PFLBM_BF16>(h, pl, steps, need); break;
+        default: e = launch_prec<PFLBM_FP16>(h, pl, steps, need); break;
     }
     if (e == cudaSuccess) {
         h->cur ^= steps & 1;
