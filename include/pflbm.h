@@ -102,9 +102,10 @@ typedef struct {
      * lattices of at least 2^21 nodes, else 1; runs of at least 16 steps
      * of a lattice that fits the chip's shared memory (up to about 270,000
      * fluid nodes in FP32, 310,000 in 16-bit storage, 75,000 in FP64) are
-     * then taken many steps per launch, the lattice held there (they
-     * allocate exchange memory on first use, which pflbm_footprint_bytes
-     * covers; without it, and on a stream under capture, the steps run one
+     * then taken many steps per launch, the lattice held there (a handle
+     * plans and allocates exchange memory, which pflbm_footprint_bytes
+     * covers, in a first run of 16 (FP64) to 64 steps, or its second run; until then,
+     * without that memory, and on a stream under capture, the steps run one
      * launch each);
      * 1: populations pulled from global memory, 32 x 8 tiles; 2:
      * populations staged in shared memory by TMA, 32 x 8 tiles; 3: staged,

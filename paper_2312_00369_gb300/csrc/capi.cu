@@ -251,6 +251,20 @@ constexpr int64_t kResidentMinSteps = 16;
 constexpr int kResidentMaxSteps = 1024;          // steps of one launch: a few milliseconds
 constexpr long long kResidentMapNodes = 1 << 20; // larger lattices never fit
 
+// On a handle that has not stepped resident yet, the plan, the count of what the lists
+// need, the memory and its clearing cost 55 to 125 us more. Measured on new handles (us,
+// single steps and resident): FP32 100 x 50 at 24 steps 137 and 131, 256 x 128 at 32
+// 185 and 174, 400 x 200 slope at 32 233 and 258, at 40 292 and 281, 512 x 512 at 50 446
+// and 468, at 64 568 and 552 (FP16 at 40 372 and 348); FP64 100 x 50 at 16 312 and 208.
+// A handle that comes back for a second run is taken to go on stepping in runs.
+bool pays_plan(pflbm_t* h, int64_t n)
+{
+    const int64_t first = h->precision == PFLBM_FP64 ? kResidentMinSteps : (long long)h->nx * h->ny <= 100000 ? 40 : 64;
+    const bool again = h->res_seen > 0;
+    h->res_seen += n;
+    return h->res_seen >= (again ? 32 : first);
+}
+
 // What a handle may allocate for them, whatever its mask.
 size_t resident_allowance(int nx, int ny, int precision)
 {
@@ -263,13 +277,14 @@ bool capturing(cudaStream_t stream)
     return cudaStreamIsCapturing(stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
 }
 
-// Whether the handle can step resident; plans and allocates on first use. A
+// Whether the handle takes n steps resident; plans and allocates on first use. A
 // stream under capture takes single steps: a replayed launch would repeat its
 // exchange tags.
-bool resident_ready(pflbm_t* h)
+bool resident_ready(pflbm_t* h, int64_t n)
 {
     if (!h->auto_kernel || h->res_state < 0 || capturing(h->stream)) return false;
     if (h->res_state > 0) return true;
+    if (!pays_plan(h, n)) return false;
     h->res_state = -1;
     int coop = 0, sms = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device);
@@ -635,7 +650,7 @@ int pflbm_step(pflbm_t* h, int64_t n)
     NvtxRange range("pflbm_step");
     if (int rc = materialize(h)) return rc;
     int64_t t = 0;
-    if (n >= kResidentMinSteps && resident_ready(h))
+    if (n >= kResidentMinSteps && resident_ready(h, n))
         if (int rc = step_resident(h, n, &t)) return rc;
     for (; t < n; ++t) {
         CK(launch_step(h));

@@ -254,6 +254,7 @@ struct pflbm {
     pfk::SolidMap map;            // lattices small enough for it only
     bool auto_kernel = true;      // the step kernel is the library's choice
     int res_state = 0;            // 0: not tried, 1: ready, -1: not for this lattice
+    int64_t res_seen = 0;         // steps of runs that could have been resident, until tried
     pfk::ResidentPlan res;
     void* res_words = nullptr;
     unsigned res_tag = 0;         // tag of the last exchange

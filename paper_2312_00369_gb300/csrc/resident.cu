@@ -52,6 +52,7 @@
 #include "step_core.cuh"
 
 #include <cmath>
+#include <cstring>
 #include <type_traits>
 
 namespace pfk {
@@ -969,20 +970,69 @@ cudaError_t launch_batch_prec(const ResidentWave& w, int cls, int nt, cudaStream
     return cudaErrorInvalidValue;
 }
 
-// Whether a patch holds a zeta = 1 node: a fluid node in it or next to it
+// Which patches of a cut hold a zeta = 1 node: a fluid node in them or next to them
 // (from the 8 x 8 blocks with fluid, so it may say yes too often, never no).
-bool patch_active(const SolidMap& m, const Rect& r, int nx)
-{
-    auto any = [&](int x0, int x1, int y0, int y1) {   // inclusive, inside the lattice
-        const int bx0 = x0 / 8, bx1 = x1 / 8 + 1, by0 = y0 / 8, by1 = y1 / 8 + 1;
-        const int s = m.bw + 1;
-        return m.sum[by1 * s + bx1] - m.sum[by0 * s + bx1] - m.sum[by1 * s + bx0] + m.sum[by0 * s + bx0] > 0;
-    };
-    const int y0 = r.y0 - 1, y1 = r.y0 + r.h;   // rows 0 and ny - 1 exist beside every patch
-    const int x0 = r.x0 - 1, x1 = r.x0 + r.w;
-    if (any(x0 < 0 ? 0 : x0, x1 >= nx ? nx - 1 : x1, y0, y1)) return true;
-    return (x0 < 0 && any(nx - 1, nx - 1, y0, y1)) || (x1 >= nx && any(0, 0, y0, y1));
-}
+// The block columns of the patches' columns (and where those reach over the
+// periodic seam) and the block rows of their rows are worked out once per px and py:
+// a plan looks at tens of thousands of patches.
+struct PatchTest {
+    struct Span { int lo, hi, seam; };     // blocks lo..hi-1; and block column `seam` (or -1)
+    const SolidMap& m;
+    int nx, unit, px = 0, py = 0;
+    std::vector<Span> cols, rows;
+    PatchTest(const SolidMap& map, int nx_, int unit_) : m(map), nx(nx_), unit(unit_) {}
+    Rect rect(const ResidentCut& c, int i) const { return unit == 1 ? patch_rect<1>(c, i, nx) : patch_rect<2>(c, i, nx); }
+    void columns(const ResidentCut& c)
+    {
+        px = c.px;
+        cols.resize(px);
+        for (int i = 0; i < px; ++i) {
+            const Rect r = rect(c, i);
+            const int x0 = r.x0 - 1, x1 = r.x0 + r.w;
+            cols[i] = {(x0 < 0 ? 0 : x0) / 8, (x1 >= nx ? nx - 1 : x1) / 8 + 1, x0 < 0 ? (nx - 1) / 8 : x1 >= nx ? 0 : -1};
+            // a single column of patches reaches over the seam at both sides, and
+            // holds both columns itself
+        }
+    }
+    void lines(const ResidentCut& c)
+    {
+        py = c.py;
+        rows.resize(py);
+        for (int j = 0; j < py; ++j) {
+            const Rect r = rect(c, j * c.px);
+            rows[j] = {(r.y0 - 1) / 8, (r.y0 + r.h) / 8 + 1, -1};   // rows 0 and ny - 1 exist beside every patch
+        }
+    }
+    bool active(int i, int j) const
+    {
+        const Span &x = cols[i], &y = rows[j];
+        const int* lo = m.sum.data() + (size_t)y.lo * (m.bw + 1);
+        const int* hi = m.sum.data() + (size_t)y.hi * (m.bw + 1);
+        if (hi[x.hi] - lo[x.hi] - hi[x.lo] + lo[x.lo] > 0) return true;
+        return x.seam >= 0 && hi[x.seam + 1] - lo[x.seam + 1] - hi[x.seam] + lo[x.seam] > 0;
+    }
+    // active patches, counted row by row of patches until they are more than cap
+    int count(int cap, int* tests) const
+    {
+        if (m.sum.back() == m.bw * m.bh) return px * py;
+        int n = 0;
+        for (int j = 0; j < py && n <= cap; ++j, *tests += px)
+            for (int i = 0; i < px; ++i) n += active(i, j);
+        return n;
+    }
+    // the set of active patches, how many lie below each of its words; their number
+    int fill(ResidentCut* c) const
+    {
+        int n = 0;
+        for (int i = 0; i < px * py; ++i) {
+            if (i % 32 == 0) c->before[i >> 5] = (uint16_t)n;
+            if (!active(i % px, i / px)) continue;
+            c->active[i >> 5] |= 1u << (i & 31);
+            ++n;
+        }
+        return n;
+    }
+};
 
 }  // namespace
 
@@ -991,31 +1041,23 @@ void SolidMap::build(const uint8_t* solid, int nx, int ny)
     bw = (nx + 7) / 8;
     bh = (ny + 7) / 8;
     sum.assign((size_t)(bw + 1) * (bh + 1), 0);
-    for (int y = 0; y < ny; ++y)
-        for (int b = 0; b < bw; ++b) {
-            int& v = sum[(size_t)(y / 8 + 1) * (bw + 1) + b + 1];
-            if (v) continue;
-            const int e = b * 8 + 8 < nx ? b * 8 + 8 : nx;
-            for (int x = b * 8; x < e; ++x)
-                if (!solid[(size_t)y * nx + x]) { v = 1; break; }
+    for (int y = 0; y < ny; ++y) {
+        const uint8_t* row = solid + (size_t)y * nx;
+        int* out = sum.data() + (size_t)(y / 8 + 1) * (bw + 1) + 1;
+        for (int b = 0; b < nx / 8; ++b) {       // a zero byte among eight
+            uint64_t v;
+            memcpy(&v, row + 8 * b, 8);
+            out[b] |= ((v - 0x0101010101010101ull) & ~v & 0x8080808080808080ull) != 0;
         }
+        for (int x = nx / 8 * 8; x < nx; ++x) out[x / 8] |= row[x] == 0;
+    }
     for (int y = 1; y <= bh; ++y)
         for (int x = 1; x <= bw; ++x)
             sum[(size_t)y * (bw + 1) + x] += sum[(size_t)(y - 1) * (bw + 1) + x] + sum[(size_t)y * (bw + 1) + x - 1] -
                                              sum[(size_t)(y - 1) * (bw + 1) + x - 1];
 }
 
-// active patches below each word of the set
-void count_before(ResidentCut* c)
-{
-    int n = 0;
-    for (int i = 0; i < kMaxPatches / 32; ++i) {
-        c->before[i] = (uint16_t)n;
-        n += __builtin_popcount(c->active[i]);
-    }
-}
-
-constexpr int kPlanTests = 30000;
+constexpr int kPlanTests = 45000;
 
 // The cut with the smallest estimated step: the collision and pulls of the
 // largest patch, and its border. Cycles per node and per border node are
@@ -1033,12 +1075,21 @@ bool plan_resident(int nx, int ny, int precision, const SolidMap& map, int max_c
     // columns of patches from the one that makes them square outwards, so that
     // most of the others are dropped by their cost alone
     const int ideal = (int)(sqrt((double)cap / fluid * nx / ny) + 0.5), most = units < kMaxPatches ? units : kMaxPatches;
-    int tests = 0;   // patches looked at; the search ends after about half a millisecond of it
+    int tests = 0;   // patches looked at; the search ends after about a tenth of a millisecond of it
+    PatchTest test(map, nx, unit);
+    const long long least = 64LL * map.sum.back() - 8LL * (nx + 8) - 8LL * (ny + 8) - 2LL * nx;   // nodes in blocks with fluid, at least
     for (int turn = 0; turn <= 2 * (ideal + most) && tests < kPlanTests; ++turn) {
         const int px = ideal + (turn & 1 ? -(turn + 1) / 2 : turn / 2);
         if (px < 1 || px > most) continue;
         const int w2 = (units + px - 1) / px * unit, lw = w2 / unit;
         if (px > 1 && lw < 4) continue;
+        ResidentCut cut{};
+        cut.px = px;
+        cut.py = 1;
+        cut.units = units;
+        cut.rows = rows;
+        cut.w = w2;
+        bool columns = false;
         for (int k = 0; k < classes(precision); ++k) {
             if (only_class >= 0 && k != only_class) continue;
             const Class c = class_of(precision, k);
@@ -1054,27 +1105,21 @@ bool plan_resident(int nx, int ny, int precision, const SolidMap& map, int max_c
                                      4.3 * 2 * (w2 + h)) *
                                     (lw == 16 ? 0.88 : lw == 32 ? 0.94 : 1.0);
                 if (cost >= best) break;      // fewer rows of patches only cost more
-                ResidentCut cut{};
-                cut.px = px;
+                // every node of a block with fluid lies in an active patch
+                if (least > (long long)cap * w2 * h) continue;
                 cut.py = py;
-                cut.units = units;
-                cut.rows = rows;
-                cut.w = w2;
                 cut.h = h;
-                int n = 0;
-                for (int i = 0; i < px * py && n <= cap; ++i, ++tests) {
-                    const Rect r = unit == 1 ? patch_rect<1>(cut, i, nx) : patch_rect<2>(cut, i, nx);
-                    if (patch_active(map, r, nx)) {
-                        cut.active[i >> 5] |= 1u << (i & 31);
-                        ++n;
-                    }
-                }
+                if (!columns) test.columns(cut);
+                columns = true;
+                test.lines(cut);
+                int n = test.count(cap, &tests);
                 if (n > cap) continue;
                 if (n == 0) break;
+                ResidentCut full = cut;
+                n = test.fill(&full);
                 best = cost;
                 found = true;
-                count_before(&cut);
-                out->cut = cut;
+                out->cut = full;
                 out->cls = k;
                 out->n_active = n;
                 const int per = ((lanes + c.p - 1) / c.p + 31) / 32 * 32;
@@ -1108,13 +1153,10 @@ bool cut_resident(int nx, int ny, int precision, const SolidMap& map, int cls, d
     cut->rows = rows;
     cut->w = (units + cut->px - 1) / cut->px * 2;
     cut->h = (rows + cut->py - 1) / cut->py;
-    int n = 0;
-    for (int i = 0; i < cut->px * cut->py; ++i)
-        if (patch_active(map, patch_rect<2>(*cut, i, nx), nx)) {
-            cut->active[i >> 5] |= 1u << (i & 31);
-            ++n;
-        }
-    count_before(cut);
+    PatchTest test(map, nx, 2);
+    test.columns(*cut);
+    test.lines(*cut);
+    const int n = test.fill(cut);
     *n_active = n;
     *half_words = (unsigned long long)n * patch_words<true>(cut->w, cut->h);
     return true;
