@@ -277,6 +277,15 @@ bool capturing(cudaStream_t stream)
     return cudaStreamIsCapturing(stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
 }
 
+// Allocating and waiting are forbidden to a thread while another captures a stream
+// in global mode (or it does so itself, another stream than the handle's), and
+// break that capture. Nothing here touches the captured stream.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // Whether the handle takes n steps resident; plans and allocates on first use. A
 // stream under capture takes single steps: a replayed launch would repeat its
 // exchange tags.
@@ -286,6 +295,7 @@ bool resident_ready(pflbm_t* h, int64_t n)
     if (h->res_state > 0) return true;
     if (!pays_plan(h, n)) return false;
     h->res_state = -1;
+    RelaxedCapture relaxed;
     int coop = 0, sms = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);

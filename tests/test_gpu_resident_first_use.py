@@ -1,6 +1,6 @@
 """A handle's first resident run: when it plans and takes its exchange memory,
-and the index-checked build over both runs of a handle. The fields equal those
-of single steps bit for bit.
+that a capture in global mode elsewhere survives it, and the index-checked build
+over both runs of a handle. The fields equal those of single steps bit for bit.
 """
 import os
 import subprocess
@@ -49,6 +49,36 @@ def test_when_a_handle_takes_exchange_memory(nx, ny, precision, runs, monkeypatc
         assert np.array_equal(a, b)
     many.close()
     one.close()
+
+
+def test_capture_elsewhere_survives_first_use():
+    """The first resident run of a handle with cudaMalloc memory, while another stream
+    is captured in global mode by the same thread: steps never allocated before resident
+    runs, so such a capture was never disturbed by them."""
+    from paper_2312_00369_gb300.pflbm import Solver
+    mine, other = torch.cuda.Stream(), torch.cuda.Stream()
+    pair = [Solver(res._frame(100, 50), precision="fp32", stream=mine, step_kernel=k, torch_memory=False)
+            for k in ("default", "global")]
+    for s in pair:
+        s.init_droplet(50.0, 0.5, 20.0)
+        s.step(1)
+    x = torch.zeros(1 << 20, device="cuda")
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=other, capture_error_mode="global"):
+        x += 1
+        pair[0].step(200)
+        x += 2
+    pair[1].step(200)
+    for _ in range(3):
+        graph.replay()
+    torch.cuda.synchronize()
+    assert bool((x == 9).all())
+    for a, b in zip(res._state(pair[0]), res._state(pair[1])):
+        assert np.array_equal(a, b)
+    del graph
+    for s in pair:
+        s.close()
 
 
 BOUNDS_SCRIPT = """
