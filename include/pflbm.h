@@ -280,8 +280,9 @@ typedef struct {
                             order and ctas_per_sm do not apply). Runs of at
                             least 16 steps take the members that fit the
                             chip's shared memory many steps per launch
-                            instead (16-bit storage, and FP32 batches of up
-                            to 2^21 nodes). FP64 batches always use 1.      */
+                            instead, where that is estimated to be faster
+                            for these members and this run. FP64 batches
+                            always use 1.                                   */
     /* Staged kernel, per size class: a lattice with nx * ny <=
      * class_max_nodes[k] (first such k < n_classes) runs with tile shape
      * class_shape[k] (0: 32 x 8, 1: 64 x 4) and class_tiles[k] tiles per
@@ -325,10 +326,11 @@ void pflbm_batch_destroy(pflbm_batch_t* b);
  * current device (0 in the normal build). Not in the paper: a test aid. */
 int pflbm_debug_bounds(int* enabled, unsigned* violations);
 /* Test aid, for one batch: *waves is the number of waves of members that a run
- * of n steps would take resident (0: launches only); refuse_after >= 0: after
+ * of n steps would take resident (0: launches only). route 0: by the estimate; 1:
+ * waves for every run of at least 16 steps; 2: never. refuse_after >= 0: after
  * that many more resident launches the next is taken as refused, as when fewer
  * SMs are to be had than the device reports (< 0: none). */
-int pflbm_debug_batch(pflbm_batch_t* b, int64_t n, int refuse_after, int* waves);
+int pflbm_debug_batch(pflbm_batch_t* b, int64_t n, int route, int refuse_after, int* waves);
 
 /* Text of the calling thread's last error ("" if none). */
 const char* pflbm_last_error(void);

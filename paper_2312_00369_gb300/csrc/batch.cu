@@ -15,11 +15,14 @@
 //
 // Runs of 16 steps and more with schedule kernel 3 or 0 step the members that
 // fit the chip's shared memory there, many steps per launch (resident.cu), in
-// waves of as many members as it holds; the rest of the batch as above.
+// waves of as many members as it holds, and the rest of the batch as above, where
+// that is estimated to be faster.
 #include <algorithm>
 #include <climits>
 #include <cstring>
+#include <set>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "pflbm_internal.cuh"
@@ -59,6 +62,9 @@ struct pflbm_batch {
     };
     std::vector<Wave> waves;
     bool no_resident = false;              // a cooperative launch was refused: launches from then on
+    int route = 0;                         // test aid: 0 by the estimate, 1 waves, 2 launches
+    double launch_us = 0, wave_us = 0;     // estimates of a step: launches; waves and the rest
+    double setup_us = 0;                   // and of the waves' set-up
     int refuse_after = -1;                 // test aid: resident launches until one is taken as refused
     std::vector<ClassLaunch> rest;
     uint4* d_items = nullptr;
@@ -232,13 +238,56 @@ int grow(pflbm_batch_t* b, void** p, size_t* cap, size_t bytes)
     return PFLBM_OK;
 }
 
-// FP32 batches of more nodes than this are left to the launches per size group,
-// which then run at 0.9 of the HBM bandwidth: measured, launches -> resident (us
-// per step) 0.20 M nodes 10.5 -> 7.1, 0.39 M 13.8 -> 12.7, 1.7 M 53.0 -> 45.4, 2.5 M
-// 62.2 -> 69.4, 10.4 M 255 -> 276. In 16-bit storage resident is faster at every
-// size: 0.20 M 10.7 -> 5.2, 0.39 M 14.2 -> 9.9, 1.7 M 48.4 -> 34.0, 2.5 M 52.1 ->
-// 48.0, 10.4 M 215 -> 186 (the launches' kernel is bound by latency there).
-constexpr long long kResidentMaxNodes32 = 1LL << 21;
+// Time of a step (us) by launches per size group and by waves, from what each has to do.
+// Launches: 64 x 8 tiles without a solid node near, with some, and without fluid;
+// groups past the four forked streams queue. A wave: what a step of its largest
+// patch takes, the exchange, and the set-up of its launch spread over the run (43 us for
+// small patches, 65 to 109 for full ones; counted low, since short runs of many
+// mixes are close and the launches' estimate errs to the low side). Fitted to 184 mixes in FP16 and FP32 (2 to 300
+// lattices of 128 x 64 to 784 x 392, flat and with obstacles, requests of many sizes),
+// runs of 200 steps: either estimate is within 12 % in nearly all. With the lines below
+// a mix runs 0.3 to 0.5 % above the faster of the two on average, at most 1 % (FP16) or
+// 6 % (FP32) above the launches. (In FP32 the lines nearly touch from 0.3 to 2 M nodes; at
+// more than 2^21 the launches run at 0.9 of the HBM bandwidth and are left alone.)
+// Measured (us a step, launches and waves): FP16 16 requests 47.5 and 33.6, 64 requests
+// 160 and 154, 256 uneven with obstacles 213 and 196, without 186 and 208, 18 of 528 x 264
+// 54.6 and 78.3; FP32 8 requests 18.8 and 13.8, 6 of 256 x 256 with a shallow slope 13.8 and
+// 12.7, 16 uneven 14.3 and 19.9, 9 of 512 x 256 33.9 and 45.4.
+struct RouteCost {
+    double fixed, plain, mixed, solid, group;   // launches
+    double wave, cycle, setup, setup_cycle;     // waves
+    double line;                                // waves below this times the launches
+    long long most;                             // nodes
+};
+constexpr RouteCost kRoute16{5.77, 8.29e-3, 19.4e-3, 4.83e-3, 0.45, 1.79, 7.49e-4, 25.0, 8e-3, 0.97, LLONG_MAX};
+constexpr RouteCost kRoute32{4.33, 10.33e-3, 18.57e-3, 8.1e-3, 0.57, 2.55, 8.52e-4, 25.0, 8e-3, 1.0, 1LL << 21};
+const RouteCost& route_cost(int precision) { return precision == PFLBM_FP32 ? kRoute32 : kRoute16; }
+
+// Estimate of a step of the members `idx` by launches.
+double launch_estimate(const pflbm_batch_t* b, const std::vector<int>& idx)
+{
+    if (idx.empty()) return 0.0;
+    const RouteCost& c = route_cost(b->precision);
+    std::set<std::pair<int, int>> sizes;
+    double us = c.fixed;
+    for (int i : idx) {
+        const pflbm_t* h = b->hs[i];
+        sizes.insert({h->nx, h->ny});
+        if (h->map.sum.empty())   // a large lattice
+            us += c.plain * ((h->nx + 63) / 64) * ((h->ny + 7) / 8);
+        else
+            us += c.plain * h->map.tiles[kTilePlain] + c.mixed * h->map.tiles[kTileMixed] + c.solid * h->map.tiles[kTileSolid];
+    }
+    return us + c.group * std::max(0, (int)sizes.size() - pflbm_batch::kForks);
+}
+
+// Whether a run of n steps takes the waves; n = 0: whether any run may.
+bool waves_pay(const pflbm_batch_t* b, int64_t n)
+{
+    if (b->route) return b->route == 1;
+    const RouteCost& c = route_cost(b->precision);
+    return b->nodes <= c.most && b->wave_us + (n ? b->setup_us / (double)n : 0.0) < c.line * b->launch_us;
+}
 
 // Waves of members stepped resident, largest members first, each into the first
 // wave with room for its patches; removes them from *idx. Where the patches
@@ -251,7 +300,6 @@ int plan_waves(pflbm_batch_t* b, std::vector<int>* idx)
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, b->device);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
     if (!coop || cls < 0 || b->no_resident) return PFLBM_OK;
-    if (b->precision == PFLBM_FP32 && b->nodes > kResidentMaxNodes32) return PFLBM_OK;
     const int n = (int)b->hs.size();
     struct Member { int i, active; ResidentCut cut; unsigned long long words; };
     auto pack = [&](double split, std::vector<Member>& ms, std::vector<int>& wave, std::vector<int>& others) {
@@ -294,6 +342,18 @@ int plan_waves(pflbm_batch_t* b, std::vector<int>* idx)
             nw = 1 + *std::max_element(wave.begin(), wave.end());
             break;
         }
+    const RouteCost& rate = route_cost(b->precision);
+    b->launch_us = launch_estimate(b, *idx);
+    b->wave_us = launch_estimate(b, others) + nw * rate.wave;
+    b->setup_us = nw * rate.setup;
+    for (int w = 0; w < nw; ++w) {
+        double most = 0;
+        for (size_t k = 0; k < ms.size(); ++k)
+            if (wave[k] == w) most = std::max(most, step_cycles(b->precision, ms[k].cut.w, ms[k].cut.h));
+        b->wave_us += rate.cycle * most;
+        b->setup_us += rate.setup_cycle * most;
+    }
+    if (!waves_pay(b, 0)) return PFLBM_OK;
     std::vector<uint4> items;
     std::vector<ResidentCut> cuts(n);
     int most = 0;
@@ -573,8 +633,8 @@ int step_launches(pflbm_batch_t* b, const std::vector<pflbm_batch::ClassLaunch>&
     return PFLBM_OK;
 }
 
-// Runs of at least this many steps take the resident path (a wave costs about
-// 20 us more than its steps), in launches of at most kResidentMaxSteps (even).
+// Runs of at least this many steps may take the resident path, in launches of at
+// most kResidentMaxSteps (even).
 constexpr int64_t kResidentMinSteps = 16;
 constexpr int kResidentMaxSteps = 1024;
 
@@ -656,7 +716,7 @@ int step_waves(pflbm_batch_t* b, int64_t n)
 // Whether a run of n steps takes the waves.
 bool runs_resident(const pflbm_batch_t* b, int64_t n)
 {
-    return !b->waves.empty() && !b->no_resident && n >= kResidentMinSteps;
+    return !b->waves.empty() && !b->no_resident && n >= kResidentMinSteps && waves_pay(b, n);
 }
 
 }  // namespace
@@ -766,10 +826,15 @@ int pflbm_batch_info(const pflbm_batch_t* b, int* n_work, int* grid, int64_t* no
     return PFLBM_OK;
 }
 
-int pflbm_debug_batch(pflbm_batch_t* b, int64_t n, int refuse_after, int* waves)
+int pflbm_debug_batch(pflbm_batch_t* b, int64_t n, int route, int refuse_after, int* waves)
 {
-    if (!b) return set_error(PFLBM_EINVAL, "batch: NULL batch");
+    if (!b || route < 0 || route > 2) return set_error(PFLBM_EINVAL, "batch: invalid arguments");
     b->refuse_after = refuse_after;
+    if (route != b->route) {
+        DeviceGuard g(b->device);
+        b->route = route;
+        if (int rc = upload(b)) return rc;
+    }
     if (waves) *waves = runs_resident(b, n) ? (int)b->waves.size() : 0;
     return PFLBM_OK;
 }

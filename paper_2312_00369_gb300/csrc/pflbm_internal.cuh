@@ -183,9 +183,12 @@ struct ResidentPlan {
     ResidentSpill room{0, 0};
     size_t bytes = 0;                   // the words and the lists' overflow
 };
-// 8 x 8 blocks with a fluid node, as a summed-area table.
+// 8 x 8 blocks with a fluid node, as a summed-area table, and how many of the 64 x 8
+// tiles have no solid node within two of them, have some, or have no fluid node.
+enum { kTilePlain = 0, kTileMixed = 1, kTileSolid = 2 };
 struct SolidMap {
     int bw = 0, bh = 0;
+    int tiles[3] = {0, 0, 0};
     std::vector<int> sum;
     void build(const uint8_t* solid, int nx, int ny);
 };
@@ -292,6 +295,7 @@ bool plan_resident(int nx, int ny, int precision, const SolidMap& map, int max_c
                    ResidentPlan* out);
 size_t resident_word_bytes();
 int resident_batch_class(int precision);              // patch class of batches; < 0: none
+double step_cycles(int precision, int w, int h);      // estimate for patches of at most w x h nodes
 // The cut of a batch's member: the fewest patches of the class (split = 1), or
 // `split` times as many rows of them. Gives its active patches and its exchange
 // words (one buffer).

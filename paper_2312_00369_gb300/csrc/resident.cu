@@ -1051,6 +1051,28 @@ void SolidMap::build(const uint8_t* solid, int nx, int ny)
         }
         for (int x = nx / 8 * 8; x < nx; ++x) out[x / 8] |= row[x] == 0;
     }
+    // kinds of 64 x 8 tiles; solid nodes of each row within two columns of a tile first
+    const int tx = (nx + 63) / 64, ty = (ny + 7) / 8;
+    std::vector<uint8_t> near((size_t)ny * tx, 0);
+    for (int y = 0; y < ny; ++y)
+        for (int i = 0; i < tx; ++i) {
+            const uint8_t* row = solid + (size_t)y * nx;
+            const int x0 = 64 * i, x1 = x0 + 64 < nx ? x0 + 64 : nx;
+            uint64_t v = 0;
+            int x = x0;
+            for (uint64_t w; x + 8 <= x1; x += 8, v |= w) memcpy(&w, row + x, 8);
+            for (; x < x1; ++x) v |= row[x];
+            for (int d = 1; d <= 2; ++d) v |= row[(x0 - d + nx) % nx] | row[(x1 + d - 1) % nx];
+            near[(size_t)y * tx + i] = v != 0;
+        }
+    for (int j = 0; j < ty; ++j)
+        for (int i = 0; i < tx; ++i) {
+            const int* f = sum.data() + (size_t)(j + 1) * (bw + 1) + 1;   // blocks, not summed yet
+            bool fluid = false, clear = j > 0 && 8 * j + 10 <= ny;
+            for (int b = 8 * i; b < 8 * i + 8 && b < bw; ++b) fluid = fluid || f[b];
+            for (int y = 8 * j - 2; clear && y < 8 * j + 10; ++y) clear = !near[(size_t)y * tx + i];
+            ++tiles[!fluid ? kTileSolid : clear ? kTilePlain : kTileMixed];
+        }
     for (int y = 1; y <= bh; ++y)
         for (int x = 1; x <= bw; ++x)
             sum[(size_t)y * (bw + 1) + x] += sum[(size_t)(y - 1) * (bw + 1) + x] + sum[(size_t)y * (bw + 1) + x - 1] -
@@ -1059,11 +1081,19 @@ void SolidMap::build(const uint8_t* solid, int nx, int ny)
 
 constexpr int kPlanTests = 45000;
 
-// The cut with the smallest estimated step: the collision and pulls of the
-// largest patch, and its border. Cycles per node and per border node are
-// measured (FP32 and 16-bit: about 2.4 and 4.3; FP64: the FP64 pipe takes 19
-// cycles a warp instruction). Rows of 16 or 32 lanes are 6 to 12 % faster than
-// others (a warp then reads whole rows: fewer bank conflicts).
+// Cycles of a step that depend on the largest patch: its collision and pulls, and
+// its border. Those per node and per border node are measured (FP32 and 16-bit:
+// about 2.4 and 4.3; FP64: the FP64 pipe takes 19 cycles a warp instruction).
+// Rows of 16 or 32 lanes are 6 to 12 % faster than others (a warp then reads
+// whole rows: fewer bank conflicts).
+double step_cycles(int precision, int w, int h)
+{
+    const int unit = precision == PFLBM_FP64 ? 1 : 2, lw = w / unit, lanes = lw * h;
+    return ((precision == PFLBM_FP64 ? 100.0 : 2.4) * ((lanes + 31) / 32 * 32 * unit) + 4.3 * 2 * (w + h)) *
+           (lw == 16 ? 0.88 : lw == 32 ? 0.94 : 1.0);
+}
+
+// The cut with the smallest estimated step.
 bool plan_resident(int nx, int ny, int precision, const SolidMap& map, int max_ctas, int only_class, ResidentPlan* out)
 {
     const int unit = precision == PFLBM_FP64 ? 1 : 2, units = (nx + unit - 1) / unit, rows = ny - 2;
@@ -1101,9 +1131,7 @@ bool plan_resident(int nx, int ny, int precision, const SolidMap& map, int max_c
             for (; py >= 1; --py) {
                 const int h = (rows + py - 1) / py, lanes = lw * h;
                 if (h > c.hm || lanes > c.p * c.nt) break;
-                const double cost = ((precision == PFLBM_FP64 ? 100.0 : 2.4) * ((lanes + 31) / 32 * 32 * unit) +
-                                     4.3 * 2 * (w2 + h)) *
-                                    (lw == 16 ? 0.88 : lw == 32 ? 0.94 : 1.0);
+                const double cost = step_cycles(precision, w2, h);
                 if (cost >= best) break;      // fewer rows of patches only cost more
                 // every node of a block with fluid lies in an active patch
                 if (least > (long long)cap * w2 * h) continue;

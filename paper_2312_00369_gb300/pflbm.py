@@ -121,7 +121,7 @@ _SIGS = {
     "pflbm_set_theta_field": (ctypes.c_int, [_H, _fp]),
     "pflbm_set_step_kernel": (ctypes.c_int, [_H, ctypes.c_int, ctypes.c_int]),
     "pflbm_debug_bounds": (ctypes.c_int, [_ip, ctypes.POINTER(ctypes.c_uint)]),
-    "pflbm_debug_batch": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int64, ctypes.c_int, _ip]),
+    "pflbm_debug_batch": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int64, ctypes.c_int, ctypes.c_int, _ip]),
     "pflbm_get_step_kernel": (ctypes.c_int, [_H]),
     "pflbm_init_droplet": (ctypes.c_int, [_H, ctypes.c_double, ctypes.c_double, ctypes.c_double]),
     "pflbm_init_phi": (ctypes.c_int, [_H, _dp]),
@@ -493,11 +493,11 @@ class Batch:
                                       ctypes.byref(nodes)))
         return dict(n_work=nw.value, grid=grid.value, nodes=nodes.value)
 
-    def debug(self, n, refuse_after=-1):
-        """Waves that a run of n steps takes resident; arms a refused launch
-        (``pflbm_debug_batch``, a test aid)."""
+    def debug(self, n, route=0, refuse_after=-1):
+        """Waves that a run of n steps takes resident; sets the route and arms a
+        refused launch (``pflbm_debug_batch``, a test aid)."""
         waves = ctypes.c_int()
-        _check(lib().pflbm_debug_batch(self._b, int(n), int(refuse_after), ctypes.byref(waves)))
+        _check(lib().pflbm_debug_batch(self._b, int(n), int(route), int(refuse_after), ctypes.byref(waves)))
         return waves.value
 
     def close(self):

@@ -44,6 +44,7 @@ def test_members_large_small_large(precision):
     many, one = _make(precision, "default", stream), _make(precision, "global", stream)
     sets = [range(6), [5], [3, 4], range(6), [4], range(6), [2, 5], [0, 1, 3]]
     b = Batch([many[i] for i in sets[0]])
+    assert b.debug(16, route=1) >= 1               # waves, whatever the estimate says
     for k, members in enumerate(sets):
         if k:
             b.set([many[i] for i in members])
@@ -81,9 +82,9 @@ def test_refused_launch_falls_back(refuse_after, before):
     b = Batch(many)
     n = 1029
     b.step(before)
-    assert b.debug(n, refuse_after) >= 2
+    assert b.debug(n, route=1, refuse_after=refuse_after) >= 2
     b.step(n)
-    assert b.debug(n) == 0
+    assert b.debug(n, route=1) == 0
     b.step(17)
     b.set(many[:3])
     b.step(20)
