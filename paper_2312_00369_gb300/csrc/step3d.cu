@@ -678,13 +678,13 @@ __global__ void k3_wet(const double* av, C* wet, size_t n, double coef)
 // this part), else in FP64. The distance is FP64 in both: the squared distance
 // along each axis is taken once per CTA, and a node costs two FP64 additions
 // (an FP64 instruction takes 19 cycles a warp and SM) where an FP32 bound does
-// not already place it outside. A CTA takes 32 x 8 columns of kDropZ planes.
+// not already place it outside. A CTA takes 32 x 8 columns of `planes` (at most kDropZ) planes.
 // Measured, 64 droplets of R 12 to 24 with W = 4: 59 us each -> 13.5 us.
 constexpr int kDropZ = 8;
 template <bool F32>
 __global__ void __launch_bounds__(256) k3_droplet(const uint8_t* __restrict__ cls, double* __restrict__ phi, int nx, int ny,
                                                   int pitch, int xlo, int xw, int ylo, int yw, int zlo, int zn, double x0,
-                                                  double y0, double z0, double R, double W, double reach)
+                                                  double y0, double z0, double R, double W, double reach, int planes)
 {
     __shared__ double s_x2[32], s_y2[8], s_z2[kDropZ];
     const int tid = threadIdx.y * 32 + threadIdx.x;
@@ -701,8 +701,8 @@ __global__ void __launch_bounds__(256) k3_droplet(const uint8_t* __restrict__ cl
     } else if (tid < 40) {
         const double d = wrap_near(node(ylo + blockIdx.y * 8 + tid - 32, ny) - y0, ny);
         s_y2[tid - 32] = d * d;
-    } else if (tid < 40 + kDropZ) {
-        const double d = (zlo + (int)blockIdx.z * kDropZ + tid - 40) - z0;
+    } else if (tid < 40 + planes) {
+        const double d = (zlo + (int)blockIdx.z * planes + tid - 40) - z0;
         s_z2[tid - 40] = d * d;
     }
     __syncthreads();
@@ -712,11 +712,11 @@ __global__ void __launch_bounds__(256) k3_droplet(const uint8_t* __restrict__ cl
     const size_t col = (size_t)node(ylo + j, ny) * pitch + node(xlo + i, nx);
     const double xy2 = s_x2[threadIdx.x] + s_y2[threadIdx.y], reach2 = reach * reach;
     const float xy2f = (float)xy2, out2f = (float)reach2 * 1.00001f;
-    for (int q = 0; q < kDropZ && blockIdx.z * kDropZ + q < zn; ++q) {
+    for (int q = 0; q < planes && (int)blockIdx.z * planes + q < zn; ++q) {
         if (xy2f + (float)s_z2[q] > out2f) continue;   // outside, whatever the last bits
         const double r2 = xy2 + s_z2[q];
         if (r2 > reach2) continue;
-        const size_t k = (size_t)(zlo + blockIdx.z * kDropZ + q) * ny * pitch + col;
+        const size_t k = (size_t)(zlo + (int)blockIdx.z * planes + q) * ny * pitch + col;
         if (!zeta_of(cls[k])) continue;
         const double v = F32 ? (double)(0.5f + 0.5f * tanhf(2.0f * ((float)R - sqrtf((float)r2)) / (float)W))
                              : 0.5 + 0.5 * tanh(2.0 * (R - sqrt(r2)) / W);
@@ -1038,10 +1038,17 @@ cudaError_t launch_ghost_flags(pflbm3d_t* h)
 cudaError_t launch_droplet(pflbm3d_t* h, int xlo, int xw, int ylo, int yw, int zlo, int zn, double x0, double y0,
                            double z0, double R, double reach)
 {
-    dim3 b(32, 8), g((xw + 31) / 32, (yw + 7) / 8, (zn + kDropZ - 1) / kDropZ);
+    // As many planes per CTA as leave every SM two CTAs: the profile of a small
+    // droplet is FP64 work (in FP64 solves) that eight planes per CTA put on a few
+    // SMs (two droplets and a step, 24 x 24 x 20 FP64, 1 plane and 8: 94 and 134 us).
+    int sms = 1, planes = kDropZ;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+    dim3 b(32, 8), g((xw + 31) / 32, (yw + 7) / 8, 1);
+    while (planes > 1 && (int)(g.x * g.y) * ((zn + planes - 1) / planes) < 2 * sms) planes /= 2;
+    g.z = (zn + planes - 1) / planes;
     auto* k = h->precision == PFLBM_FP64 ? k3_droplet<false> : k3_droplet<true>;
     return launch_after(k, g, b, h->stream, (const uint8_t*)h->cls, h->phi0, h->nx, h->ny, h->pitch, xlo, xw, ylo, yw, zlo, zn,
-                        x0, y0, z0, R, h->prm.W, reach);
+                        x0, y0, z0, R, h->prm.W, reach, planes);
 }
 
 cudaError_t fused_setup(int precision, size_t* smem_bytes, int* ctas_per_sm)
