@@ -6,14 +6,16 @@ The batched step has three kernels and several knobs (``pflbm_schedule_t``):
   tile column per work item, item order;
 * the two-node kernel (64 x 8 tiles, two x-adjacent nodes per thread in
   packed FP32x2 arithmetic; one launch per group of same-size lattices,
-  side by side): no knobs, one candidate;
+  side by side, or for runs of at least 16 steps members held in shared memory
+  where the library finds that faster): no knobs, one candidate;
 * the staged kernel (TMA ring): per size class of the mix, the tile shape
   (32 x 8 or 64 x 4) and the tiles a CTA marches down per work item.
 
 The best choice depends on the mix of lattice sizes and on the GPU, so it is
-measured. Every candidate runs a few batched steps on scratch copies of the
+measured. Every candidate runs batched steps on scratch copies of the
 lattices (same geometry and parameters, so the real solves are not
-advanced), timed with CUDA events. The global-load kernel's knobs are
+advanced), timed with CUDA events: a run as long as those to come (200 steps by
+default), since a shorter one would not see what the two-node schedule does then. The global-load kernel's knobs are
 swept as a grid; the staged kernel's per-class shape and item length are
 chosen by coordinate descent over the classes, largest total node count
 first. The fastest schedule is cached per (GPU, precision, size mix) in a
@@ -42,7 +44,7 @@ def cache_path():
 def signature(cases, precision, device_name):
     sizes = sorted((int(c.nx), int(c.ny)) for c in cases)
     h = hashlib.sha1(json.dumps(sizes).encode()).hexdigest()[:16]
-    return f"v4|{device_name}|{precision}|{len(sizes)}|{h}"
+    return f"v5|{device_name}|{precision}|{len(sizes)}|{h}"
 
 
 def _load_cache():
@@ -80,9 +82,10 @@ def to_schedule(sched):
     return pflbm.schedule(classes=[tuple(c) for c in sched.get("classes", [])], **kw)
 
 
-def tune(cases, precision="bf16", stream=None, steps=12, warmup=4, candidates=None,
+def tune(cases, precision="bf16", stream=None, steps=200, warmup=16, candidates=None,
          use_cache=True, verbose=False, staged=True):
-    """Return (best schedule dict, {candidate name: ms per step}) for the cases."""
+    """Return (best schedule dict, {candidate name: ms per step}) for the cases and
+    runs of ``steps`` steps."""
     import torch
     dev = torch.cuda.current_device()
     key = signature(cases, precision, torch.cuda.get_device_name(dev))
