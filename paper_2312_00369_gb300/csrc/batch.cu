@@ -633,17 +633,6 @@ int step_launches(pflbm_batch_t* b, const std::vector<pflbm_batch::ClassLaunch>&
     return PFLBM_OK;
 }
 
-// Runs of at least this many steps may take the resident path, in launches of at
-// most kResidentMaxSteps (even).
-constexpr int64_t kResidentMinSteps = 16;
-constexpr int kResidentMaxSteps = 1024;
-
-bool capturing(cudaStream_t stream)
-{
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    return cudaStreamIsCapturing(stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
-}
-
 // A resident launch; cudaErrorCooperativeLaunchTooLarge and the like when fewer
 // SMs are to be had than the device reports.
 cudaError_t launch_wave(pflbm_batch_t* b, const ResidentWave& a, int cls)

@@ -240,15 +240,13 @@ int select_step_kernel(pflbm_t* h, int kernel, int chunk)
     return PFLBM_OK;
 }
 
-// Runs of at least this many steps are taken resident where the lattice fits
+// Runs of at least kResidentMinSteps are taken resident where the lattice fits
 // (resident.cu), when the step kernel is the library's choice. A resident
 // launch takes 16 to 60 us before its first step (cooperative launch, loading
 // the state, its lists). Measured, 16 single steps and 16 resident (us): FP32
 // 100 x 50 82 and 50, 256 x 128 92 and 66, 400 x 200 106 and 98, 512 x 512 155 and
 // 159 (at 32 steps 310 and 253); BF16 512 x 512 159 and 127; FP64 100 x 50 300
 // and 123, 256 x 128 271 and 247.
-constexpr int64_t kResidentMinSteps = 16;
-constexpr int kResidentMaxSteps = 1024;          // steps of one launch: a few milliseconds
 constexpr long long kResidentMapNodes = 1 << 20; // larger lattices never fit
 
 // On a handle that has not stepped resident yet, the plan, the count of what the lists
@@ -271,12 +269,6 @@ size_t resident_allowance(int nx, int ny, int precision)
     return (long long)nx * ny <= kResidentMapNodes ? resident_bytes_at_most(nx, ny, precision) : 0;
 }
 
-bool capturing(cudaStream_t stream)
-{
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    return cudaStreamIsCapturing(stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
-}
-
 // Allocating and waiting are forbidden to a thread while another captures a stream
 // in global mode (or it does so itself, another stream than the handle's), and
 // break that capture. Nothing here touches the captured stream.
@@ -296,10 +288,9 @@ bool resident_ready(pflbm_t* h, int64_t n)
     if (!pays_plan(h, n)) return false;
     h->res_state = -1;
     RelaxedCapture relaxed;
-    int coop = 0, sms = 0;
+    int coop = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-    if (!coop || !plan_resident(h->nx, h->ny, h->precision, h->map, sms, -1, &h->res)) return false;
+    if (!coop || !plan_resident(h->nx, h->ny, h->precision, h->map, (int)h->sms, -1, &h->res)) return false;
     // what the lists need past shared memory (nothing, but for dense obstacles):
     // dstatus[2..3] and hstatus[2..3] are for this alone
     h->res_tag = 0;
@@ -439,6 +430,9 @@ int pflbm_create_ex(pflbm_t** out, const pflbm_params_t* prm)
     }
     h->device = dev;
     DeviceGuard guard(dev);
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    h->sms = (unsigned)sms;
     // derived parameters (Eqs. b1, initialphi, mobility)
     Params& q = h->prm;
     q.sigma = prm->sigma;

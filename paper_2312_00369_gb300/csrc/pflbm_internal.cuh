@@ -192,6 +192,17 @@ struct SolidMap {
     std::vector<int> sum;
     void build(const uint8_t* solid, int nx, int ny);
 };
+// Runs of at least this many steps may be taken resident, in launches of at most
+// kResidentMaxSteps (even; a few milliseconds).
+constexpr int64_t kResidentMinSteps = 16;
+constexpr int kResidentMaxSteps = 1024;
+// Whether a stream is being captured (or cannot say).
+inline bool capturing(cudaStream_t stream)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
+}
+
 // One launch over patches of several lattices.
 struct ResidentWave {
     const void* args;                   // step descriptors (device)
@@ -256,6 +267,7 @@ struct pflbm {
     // resident steps (resident.cu): plan and exchange words, made on first use
     pfk::SolidMap map;            // lattices small enough for it only
     bool auto_kernel = true;      // the step kernel is the library's choice
+    unsigned sms = 0;             // the device's SMs
     int res_state = 0;            // 0: not tried, 1: ready, -1: not for this lattice
     int64_t res_seen = 0;         // steps of runs that could have been resident, until tried
     pfk::ResidentPlan res;

@@ -610,11 +610,11 @@ cudaError_t run_step_kernel(pflbm_t* h, double* o_phi, double* o_u, double* o_p,
     a.f_u = f_u;
     a.f_p = f_p;
     dim3 b(TX, TY), g(tiles_x(h->nx), tiles_y(h->ny));
-    // An FP64 step of less than a wave (3 CTAs on each of 152 SMs) launches after
+    // An FP64 step of less than a wave (3 CTAs on each SM) launches after
     // the one before it: started early, its CTAs crowd the SMs that the other
     // grid leaves free, and the FP64 pipe is what bounds them (256 x 128: 16.5
     // us a step, 35.7 started early; 350 x 300, just below a wave, 41.1 and 38.2).
-    if (PREC == PFLBM_FP64 && g.x * g.y < 3 * 152) {
+    if (PREC == PFLBM_FP64 && g.x * g.y < 3u * h->sms) {
         if (a.varvisc)
             k_step<PREC, COLLIDE, 1><<<g, b, 0, h->stream>>>(a);
         else
