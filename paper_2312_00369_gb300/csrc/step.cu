@@ -53,9 +53,11 @@ namespace {
 // k_step takes the rows of larger FP32 lattices up and down in turn (the copy
 // read says which), so that a step begins with what L2 (129 MB) still holds of
 // the rows written last. Measured, us a step (in brackets what a step reads and
-// writes), always up and in turn: 1021 x 383 (59 MB) 11.6 and 11.9, 1024 x 768
-// (120 MB) 24.6 and 22.4, 1024 x 1024 (159 MB) 31.8 and 29.0, 1500 x 1000 (228 MB) 40.5
-// and 38.8. From 2^21 nodes k_step2 is the default. The direction is a template
+// writes), always up and in turn: 1021 x 383 (59 MB) 11.0 and 11.2, 1021 x 450 (70 MB)
+// 11.9 and 12.3, 800 x 640 (78 MB) 13.7 and 14.1, 860 x 640 (84 MB) 15.2 and 15.4, 900 x
+// 700 (96 MB) 18.7 and 18.2, 1000 x 700 (106 MB) 21.2 and 20.0, 1024 x 768 (120 MB) 24.2
+// and 21.7, 1024 x 1024 (159 MB) 31.8 and 29.0, 1500 x 1000 (228 MB) 40.5 and 38.8. From
+// 2^21 nodes k_step2 is the default. The direction is a template
 // argument: read from the descriptor it cost the other lattices 0.5 to 1 %.
 // (k_step2 with it as a template argument lost 3 to 12 %, the overlap of its
 // launches; read from the descriptor it gained 0.5 to 11 % where L2 holds a part
@@ -63,7 +65,7 @@ namespace {
 bool rows_down(const pflbm_t* h)
 {
     const double nodes = (double)h->nx * h->ny;
-    return h->cur && h->precision == PFLBM_FP32 && 152.0 * nodes > 64e6 && nodes < (double)(1 << 21);
+    return h->cur && h->precision == PFLBM_FP32 && 152.0 * nodes > 90e6 && nodes < (double)(1 << 21);
 }
 
 // Prologue of a tile whose nodes within two of it are all fluid: no class
