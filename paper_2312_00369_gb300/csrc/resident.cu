@@ -10,9 +10,9 @@
 //
 // Measured (us per step in runs of 1000, one launch per step -> resident; the
 // launches in brackets overlap their heads and tails, launch_after):
-// FP32 100 x 50 6.16 (5.1) -> 2.04, 256 x 128 6.17 (5.8) -> 2.42, 400 x 200 with
-// a 30 degree slope 8.21 (6.6) -> 2.83, 512 x 512 with a disc 10.3 (9.7) -> 5.9
-// (BF16 10.7 (9.9) -> 5.0); FP64 100 x 50 18.4 -> 6.1, 400 x 200 41.0 -> 18.2. What a step of 256 x 128
+// FP32 100 x 50 6.16 (5.1) -> 1.92, 256 x 128 6.17 (5.8) -> 2.34, 400 x 200 with
+// a 30 degree slope 8.21 (6.6) -> 2.65, 512 x 512 with a disc 10.3 (9.7) -> 5.9
+// (BF16 10.7 (9.9) -> 4.9); FP64 100 x 50 18.4 -> 6.1, 400 x 200 41.0 -> 18.2. What a step of 256 x 128
 // takes (cycles, a patch at the wall): bounce-back copies, pulls and phi
 // 1,100, ghost values 800, collision 1,000, publishing 400, the wait 1,650. With
 // larger patches the pulls (shared-memory bandwidth) and the collision (FP32
@@ -1198,10 +1198,11 @@ ResidentSpill resident_spill(int precision, int cls)
     return cls == 0 ? spill_k<PFLBM_BF16, 0>() : cls == 1 ? spill_k<PFLBM_BF16, 1>() : spill_k<PFLBM_BF16, 2>();
 }
 
-// The overflow that a handle's footprint allows for: 32-bit words per patch, an
-// eighth of its exchange words' memory. Dense obstacles need it: 5 x 5 solid
-// blocks every 8 nodes take about 900 of a 64 x 32 patch's 2304.
-static int spill_allowed(int w, int h) { return 24 * (w + h); }
+// The overflow that a handle's footprint allows for: 32-bit words per patch, a third
+// of its exchange words' memory. Dense obstacles need it: 5 x 5 solid blocks every 8
+// nodes take about 900 of a 64 x 32 patch's 5760, single fluid nodes every 4 nodes,
+// which have the most links a mask can have, about 4600 of a 52 x 34 patch's 5160.
+static int spill_allowed(int w, int h) { return 60 * (w + h); }
 
 bool add_spill(ResidentPlan* pl, const int need[2])
 {

@@ -2,7 +2,8 @@
 exchange memory of resident runs and the FP64 read-back's scratch included, for
 any mask; and the runs that use that memory equal single steps bit for bit.
 Masks: open channel, disc, dense blocks (whose exchange lists overflow shared
-memory), one-node slits, a corridor that fills a corner of a large lattice.
+memory), one-node slits and pores (the most links), a corridor that fills a
+corner of a large lattice.
 """
 import numpy as np
 import pytest
@@ -34,8 +35,14 @@ def _corner(nx, ny):
     return s
 
 
-MASKS = {"frame": _frame, "disc": _disc, "dense3": lambda a, b: dense(a, b, 3, 6), "dense5": lambda a, b: dense(a, b, 5, 8),
-         "slits": _slits, "corner": _corner}
+def _pores(nx, ny):
+    s = np.ones((ny, nx), np.uint8)
+    s[3:-3:4, 1::4] = 0
+    return s
+
+
+MASKS = {"frame": _frame, "disc": _disc, "dense3": lambda a, b: dense(a, b, 3, 6),
+         "dense5": lambda a, b: dense(a, b, 5, 8), "slits": _slits, "pores": _pores, "corner": _corner}
 SIZES = [(3, 5), (64, 32), (100, 50), (129, 65), (256, 128), (400, 200), (512, 512), (1000, 700)]
 
 
