@@ -242,8 +242,8 @@ int select_step_kernel(pflbm_t* h, int kernel, int chunk)
 
 // Runs of at least kResidentMinSteps are taken resident where the lattice fits
 // (resident.cu), when the step kernel is the library's choice. A resident
-// launch takes 16 to 60 us before its first step (cooperative launch, loading
-// the state, its lists). Measured, 16 single steps and 16 resident (us): FP32
+// launch takes 30 to 75 us before its first step (cooperative launch, loading
+// the state, its lists). Measured on a handle that has stepped so, 16 single steps and 16 resident (us): FP32
 // 100 x 50 82 and 50, 256 x 128 92 and 66, 400 x 200 106 and 98, 512 x 512 155 and
 // 159 (at 32 steps 310 and 253); BF16 512 x 512 159 and 127; FP64 100 x 50 300
 // and 123, 256 x 128 271 and 247.

@@ -3,7 +3,8 @@
 Requests (grid size, wall type, contact angle, step count) arrive over time.
 The server keeps every admitted solve resident on the device and admits
 queued requests, first come first served, as soon as their HBM footprint
-(``pflbm_footprint_bytes``) fits the budget and a slot is free. All resident
+(``pflbm_footprint_bytes``) fits the budget and a slot is free (the batch's own
+buffers, at most 50 MB whatever its members, come on top). All resident
 solves advance together in ticks of up to ``tick`` steps: one persistent
 launch per step over every resident lattice (``pflbm_batch_t``), so requests
 that arrive while others run share the device with them. A solve whose
