@@ -243,11 +243,11 @@ int grow(pflbm_batch_t* b, void** p, size_t* cap, size_t bytes)
 // groups past the four forked streams queue. A wave: what a step of its largest
 // patch takes, the exchange, and the set-up of its launch spread over the run (43 us for
 // small patches, 65 to 109 for full ones; counted low, since short runs of many
-// mixes are close and the launches' estimate errs to the low side). Fitted to 184 mixes in FP16 and FP32 (2 to 300
-// lattices of 128 x 64 to 784 x 392, flat and with obstacles, requests of many sizes),
-// runs of 200 steps: either estimate is within 12 % in nearly all. With the lines below
-// a mix runs 0.3 to 0.5 % above the faster of the two on average, at most 1 % (FP16) or
-// 6 % (FP32) above the launches. (In FP32 the lines nearly touch from 0.3 to 2 M nodes; at
+// mixes are close and the launches' estimate errs to the low side). Fitted to 184 mixes
+// in FP16 and FP32 (2 to 300 lattices of 128 x 64 to 784 x 392, flat and with obstacles,
+// requests of many sizes), runs of 200 steps: either estimate is within 12 % in nearly
+// all. With the lines below a mix runs 0.3 to 0.5 % above the faster of the two on
+// average, at most 1 % (FP16) or 6 % (FP32) above the launches. (In FP32 the lines nearly touch from 0.3 to 2 M nodes; at
 // more than 2^21 the launches run at 0.9 of the HBM bandwidth and are left alone.)
 // Measured (us a step, launches and waves): FP16 16 requests 47.5 and 33.6, 64 requests
 // 160 and 154, 256 uneven with obstacles 213 and 196, without 186 and 208, 18 of 528 x 264
@@ -299,7 +299,8 @@ int plan_waves(pflbm_batch_t* b, std::vector<int>* idx)
     int coop = 0, sms = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, b->device);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
-    if (!coop || cls < 0 || b->no_resident) return PFLBM_OK;
+    if (!coop || cls < 0 || b->no_resident || b->route == 2) return PFLBM_OK;
+    if (!b->route && b->nodes > route_cost(b->precision).most) return PFLBM_OK;
     const int n = (int)b->hs.size();
     struct Member { int i, active; ResidentCut cut; unsigned long long words; };
     auto pack = [&](double split, std::vector<Member>& ms, std::vector<int>& wave, std::vector<int>& others) {
