@@ -281,6 +281,7 @@ def batched_line(args, torch, world, local, steps, warmup, plain=True, precision
         sv.check()
     info = b.info()
     kernel = b.kernel
+    waves = b.debug(steps)
     b.close()
     for sv in solvers:
         sv.close()
@@ -320,19 +321,19 @@ def batched_line(args, torch, world, local, steps, warmup, plain=True, precision
         "plain_fp32_one_launch_per_lattice_mlups": plain_mlups,
         "speedup_vs_plain": (value / plain_mlups) if plain_mlups else None,
         "autotune_ms_per_step": timings,
-        "gpu_launches": batched_launches(kernel, info["grid"], nodes, steps), "clocks": clocks,
+        "gpu_launches": batched_launches(kernel, info["grid"], waves, steps), "clocks": clocks,
     }
 
 
-def batched_launches(kernel, grid, nodes, steps):
+def batched_launches(kernel, grid, waves, steps):
     """Step kernels launched by a batched run, at least. The two-node kernel
     runs one launch per group of same-size lattices each step (batch info's
-    grid), the others one launch a step. Runs of 16 steps and more may go
-    through the resident kernel instead: waves of at most 152 patches of at
-    most 2048 nodes, each wave one launch per 1024 steps."""
-    if kernel == 2 or steps < 16:
-        return (grid if kernel == 3 else 1) * steps
-    return -(-nodes // (152 * 2048)) * -(-steps // 1024)
+    grid), the others one launch a step. Where the run goes by waves of members
+    held in shared memory, each wave is one launch per 1024 steps (members that
+    do not fit are launched per step as before)."""
+    if waves:
+        return waves * -(-steps // 1024)
+    return (grid if kernel == 3 else 1) * steps
 
 
 def run_serving(args, torch, rank, world, local):
