@@ -314,7 +314,7 @@ int pflbm_batch_step(pflbm_batch_t* b, int64_t n);
 int pflbm_batch_kernel(const pflbm_batch_t* b);
 /* Work items, persistent grid size and total nodes of the batch (kernel 3:
  * the CTAs of all launches, one 64 x 8 tile each, and the number of
- * launches per step). */
+ * launches per step; of the launches also where a run may go resident). */
 int pflbm_batch_info(const pflbm_batch_t* b, int* n_work, int* grid, int64_t* nodes);
 void pflbm_batch_destroy(pflbm_batch_t* b);
 
