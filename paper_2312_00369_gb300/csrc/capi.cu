@@ -152,6 +152,7 @@ void release(pflbm_t* h)
     dfree(h, h->nword, node_words_bytes(h->nx, h->ny));
     dfree(h, h->tiles2, tile2_flags_bytes(h->nx, h->ny));
     dfree(h, h->res_words, h->res.bytes);
+    dfree(h, h->res_spill, h->res.spill_bytes);
     if (h->hstatus) cudaFreeHost(h->hstatus);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
     delete h;
@@ -250,10 +251,10 @@ int select_step_kernel(pflbm_t* h, int kernel, int chunk)
 constexpr long long kResidentMapNodes = 1 << 20; // larger lattices never fit
 
 // On a handle that has not stepped resident yet, the plan, the count of what the lists
-// need, the memory and its clearing cost 55 to 125 us more. Measured on new handles (us,
-// single steps and resident): FP32 100 x 50 at 24 steps 137 and 131, 256 x 128 at 32
-// 185 and 174, 400 x 200 slope at 32 233 and 258, at 40 292 and 281, 512 x 512 at 50 446
-// and 468, at 64 568 and 552 (FP16 at 40 372 and 348); FP64 100 x 50 at 16 312 and 208.
+// need, the memory and its clearing cost 40 to 90 us more. Measured on new handles (us,
+// single steps and resident): FP32 100 x 50 at 24 steps 137 and 131, 256 x 128 at 40 224
+// and 185, 400 x 200 slope at 40 292 and 252, 512 x 512 at 50 446 and 468, at 64 568 and
+// 516 (FP16 at 40 372 and 348); FP64 100 x 50 at 16 312 and 201.
 // A handle that comes back for a second run is taken to go on stepping in runs.
 bool pays_plan(pflbm_t* h, int64_t n)
 {
@@ -291,24 +292,31 @@ bool resident_ready(pflbm_t* h, int64_t n)
     int coop = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device);
     if (!coop || !plan_resident(h->nx, h->ny, h->precision, h->map, (int)h->sms, -1, &h->res)) return false;
-    // what the lists need past shared memory (nothing, but for dense obstacles):
-    // dstatus[2..3] and hstatus[2..3] are for this alone
+    // without memory for it, single steps: they need no more
+    auto take = [&](size_t bytes) -> void* {
+        void* p = nullptr;
+        if (h->alloc_fn) p = h->alloc_fn(bytes, h->alloc_ctx);
+        else if (cudaMalloc(&p, bytes) != cudaSuccess) { cudaGetLastError(); p = nullptr; }
+        if (p) h->bytes_allocated += bytes;
+        return p;
+    };
+    // A launch of 0 steps counts what the lists need past shared memory (nothing, but
+    // for dense obstacles); the words are taken and cleared meanwhile. dstatus[2..3]
+    // and hstatus[2..3] are for this alone.
     h->res_tag = 0;
-    if (cudaMemsetAsync(h->dstatus + 2, 0, 2 * sizeof(int), h->stream) != cudaSuccess ||
-        launch_resident(h, h->res, 0, h->dstatus + 2) != cudaSuccess ||
-        cudaMemcpyAsync(h->hstatus + 2, h->dstatus + 2, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
-        cudaStreamSynchronize(h->stream) != cudaSuccess) {
+    const bool counted =
+        cudaMemsetAsync(h->dstatus + 2, 0, 2 * sizeof(int), h->stream) == cudaSuccess &&
+        launch_resident(h, h->res, 0, h->dstatus + 2) == cudaSuccess &&
+        cudaMemcpyAsync(h->hstatus + 2, h->dstatus + 2, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream) == cudaSuccess &&
+        (h->res_words = take(h->res.bytes)) != nullptr &&
+        cudaMemsetAsync(h->res_words, 0, h->res.bytes, h->stream) == cudaSuccess &&
+        cudaStreamSynchronize(h->stream) == cudaSuccess;
+    if (!counted) {
         cudaGetLastError();
         return false;
     }
     if (!add_spill(&h->res, h->hstatus + 2)) return false;
-    void* p = nullptr;
-    if (h->alloc_fn) p = h->alloc_fn(h->res.bytes, h->alloc_ctx);
-    else if (cudaMalloc(&p, h->res.bytes) != cudaSuccess) { cudaGetLastError(); p = nullptr; }
-    if (!p) return false;                        // single steps need no more memory
-    h->bytes_allocated += h->res.bytes;
-    h->res_words = p;
-    if (cudaMemsetAsync(p, 0, h->res.bytes, h->stream) != cudaSuccess) { cudaGetLastError(); return false; }
+    if (h->res.spill_bytes && !(h->res_spill = take(h->res.spill_bytes))) return false;
     h->res_state = 1;
     return true;
 }
@@ -320,7 +328,7 @@ int step_resident(pflbm_t* h, int64_t n, int64_t* done)
     while (*done < n) {
         const int c = (int)std::min<int64_t>(n - *done, kResidentMaxSteps);
         if (h->res_tag > UINT32_MAX - 2u * kResidentMaxSteps) {   // tags start again
-            CK(cudaMemsetAsync(h->res_words, 0, h->res.words * resident_word_bytes(), h->stream));
+            CK(cudaMemsetAsync(h->res_words, 0, h->res.bytes, h->stream));
             h->res_tag = 0;
         }
         if (launch_resident(h, h->res, c) != cudaSuccess) {

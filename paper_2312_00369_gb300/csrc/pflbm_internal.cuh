@@ -181,7 +181,7 @@ struct ResidentPlan {
     int cls = 0, nt = 0, n_active = 0;  // patch class, threads per CTA, CTAs
     unsigned long long words = 0;       // exchange words (both buffers)
     ResidentSpill room{0, 0};
-    size_t bytes = 0;                   // the words and the lists' overflow
+    size_t bytes = 0, spill_bytes = 0;  // of the words; of the lists' overflow
 };
 // 8 x 8 blocks with a fluid node, as a summed-area table, and how many of the 64 x 8
 // tiles have no solid node within two of them, have some, or have no fluid node.
@@ -271,7 +271,7 @@ struct pflbm {
     int res_state = 0;            // 0: not tried, 1: ready, -1: not for this lattice
     int64_t res_seen = 0;         // steps of runs that could have been resident, until tried
     pfk::ResidentPlan res;
-    void* res_words = nullptr;
+    void *res_words = nullptr, *res_spill = nullptr;
     unsigned res_tag = 0;         // tag of the last exchange
 };
 
@@ -317,7 +317,7 @@ ResidentSpill resident_spill(int precision, int cls);   // room per CTA of a bat
 // Takes the overflow that a launch of 0 steps found into the plan; false: more
 // than a handle's footprint allows for.
 bool add_spill(ResidentPlan* plan, const int need[2]);
-// Upper bound of ResidentPlan::bytes for any mask of this size.
+// Upper bound of a plan's words and overflow for any mask of this size.
 size_t resident_bytes_at_most(int nx, int ny, int precision);
 cudaError_t launch_resident_wave(int precision, const ResidentWave& w, int cls, cudaStream_t stream);
 // (steps = 0: only the largest overflow of a list and of the copies, into need[0..1])

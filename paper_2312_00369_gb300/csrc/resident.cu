@@ -62,6 +62,9 @@ namespace {
 // us and more), so some seconds; in a healthy run a word is there within a step.
 constexpr int kSpinLimit = 1 << 22;
 constexpr int kHaloX = 4, kHaloY = 3;   // three nodes are read; four in x keeps pairs aligned
+// patches that a halo of three reaches, at most: one of three nodes or more at
+// each side, three of one row above and below
+constexpr int kMostHeartbeats = 3 * 7 - 1;
 constexpr int kMaxResident = 152;       // CTAs of a one-lattice launch at most (one per SM)
 
 // A word of the exchange: three 32-bit payloads and the step tag, one 128-bit
@@ -550,6 +553,21 @@ __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ R
         if (!own && want) sRing[atomicAdd(&s_n[2], 1)] = (uint16_t)c;
     }
     __syncthreads();
+    if constexpr (!BATCH) {
+        if (q.steps == 0) {                       // only the lists' lengths
+            for (int c = tid; c < area; c += NT) {
+                const int ly = c / rs - kHaloY, lx = c % rs - kHaloX, n = __popc(mask[c]);
+                if (n) atomicAdd(&s_n[lx >= 0 && lx < r.w && ly >= 0 && ly < r.h], n);
+            }
+            __syncthreads();
+            if (tid == 0) {
+                const int poll = s_n[0] + kMostHeartbeats;
+                atomicMax(&q.need[0], (poll > s_n[1] ? poll : s_n[1]) - L::CAP);
+                atomicMax(&q.need[1], s_n[4] - L::COPIES);
+            }
+            return;
+        }
+    }
     for (int p = 0; p < kTypes; ++p) {
         for (int c0 = tid & ~31; c0 < area; c0 += NT) {
             const int c = c0 + (tid & 31), ly = c / rs - kHaloY, lx = c % rs - kHaloX;
@@ -610,15 +628,6 @@ __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ R
     __syncthreads();
     for (int c = tid; c < area; c += NT) sPhi[c] = R(0);
     const int n_poll = s_n[0], n_pub = s_n[1], n_ring = s_n[2], n_ghost = s_n[3], n_copy = s_n[4];
-    if constexpr (!BATCH) {
-        if (q.steps == 0) {
-            if (tid == 0) {
-                atomicMax(&q.need[0], (n_poll > n_pub ? n_poll : n_pub) - L::CAP);
-                atomicMax(&q.need[1], n_copy - L::COPIES);
-            }
-            return;
-        }
-    }
     if (n_poll > room_list || n_pub > room_list || n_copy > room_copy) {   // cannot happen (the room was worked out); nothing was written past the lists
         if (tid == 0) atomicOr(a.status, 4);
         return;
@@ -935,7 +944,7 @@ cudaError_t launch_prec(pflbm_t* h, const ResidentPlan& pl, int steps, int* need
     q.cut = pl.cut;
     q.ll = (Word*)h->res_words;
     q.ll_half = pl.words / 2;
-    q.spill = (uint32_t*)(q.ll + pl.words);
+    q.spill = (uint32_t*)h->res_spill;
     q.room = pl.room;
     q.need = need;
     q.tag = h->res_tag;
@@ -1208,7 +1217,7 @@ bool add_spill(ResidentPlan* pl, const int need[2])
 {
     pl->room = {need[0] > 0 ? need[0] : 0, need[1] > 0 ? need[1] : 0};
     if (pl->room.words() > spill_allowed(pl->cut.w, pl->cut.h)) return false;
-    pl->bytes = pl->words * sizeof(Word) + (size_t)pl->n_active * pl->room.words() * 4;
+    pl->spill_bytes = (size_t)pl->n_active * pl->room.words() * 4;
     return true;
 }
 
