@@ -130,9 +130,10 @@ __host__ __device__ __forceinline__ Rect patch_rect(const ResidentCut& c, int id
 // that crosses horizontal borders takes rows of nodes, one that crosses
 // vertical ones columns: of f the outermost at each side (what a pull reaches),
 // of g the three outermost (a pull on the ring of one, or of two next to a
-// ghost), so 24 (w + h) words in all. Words of nodes side by side lie side by
-// side, three columns' as rows of three (column after column a step of 512 x 512
-// FP32 took 5.99 us instead of 5.79).
+// ghost), so 24 (w + h) words in all. The words of a row lie side by side, those of
+// the columns at both sides too: a warp publishes them together (400 steps of 256 x
+// 128 FP32: the two sides apart 956 us, together 922; column after column 512 x 512
+// FP32 took 3.5 % more).
 // ROOMY (batches, whose words are one buffer however many the members): the place
 // among the type's, each of which takes all 6 (w + h) border nodes, rows first.
 // With the compact places a step of 256 uneven lattices in BF16 took 179 us
@@ -144,8 +145,8 @@ __device__ __forceinline__ int slot_of(const ResidentCut& c, const Rect& r, int 
     if (ROOMY) return ly < 3 || ly >= r.h - 3 ? row * r.w + lx : 6 * r.w + ly * 6 + col;
     const int tt = t % 6, g = 6 * (c.w + c.h);
     if (tt < 3) return t < 6 ? (2 * tt + (ly != 0)) * c.w + lx : g + (6 * tt + row) * c.w + lx;
-    if (t < 6) return 6 * c.w + (2 * (tt - 3) + (lx != 0)) * c.h + ly;
-    return g + 18 * c.w + (6 * (tt - 3) + (lx < 3 ? 0 : 3)) * c.h + 3 * ly + col % 3;
+    if (t < 6) return 6 * c.w + 2 * (tt - 3) * c.h + 2 * ly + (lx != 0);
+    return g + 18 * c.w + 6 * (tt - 3) * c.h + 6 * ly + col;
 }
 
 // Words of a patch in one buffer: its types' places, then the heartbeat in a line
@@ -218,7 +219,7 @@ template <int PREC> struct ResArgs<PREC, false> : ResCommon {
     StepArgs<PREC> a;
     ResidentCut cut;
     ResidentSpill room;              // of each CTA in spill (batches: Lay::kMost)
-    int* need;                       // steps = 0: only the largest overflow of a list and of the copies
+    int* need;                       // COUNT: the largest overflow of a list and of the copies
     uint16_t item[kMaxResident];     // patch of each CTA
 };
 template <int PREC> struct ResArgs<PREC, true> : ResCommon {
@@ -382,7 +383,8 @@ struct LaneS {
     }
 };
 
-template <int PREC, int VV, int WM, int HM, int P, int NTMAX, bool BATCH>
+// COUNT: only the lengths of the lists, into need.
+template <int PREC, int VV, int WM, int HM, int P, int NTMAX, bool BATCH, bool COUNT>
 __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ ResArgs<PREC, BATCH> q)
 {
     using T = Store<PREC>;
@@ -477,7 +479,7 @@ __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ R
         const int k = in ? gy * pitch + wrapn(r.x0 + lx, nx) : 0;
         sW[c] = in ? PFLBM_LD(a.cls, k, plane) : (uint8_t)CLS_OUT;
         mask[c] = 0;
-        if (!BATCH && q.steps == 0) continue;
+        if constexpr (COUNT) continue;
         sG0[c] = in ? PFLBM_LD(a.in.g0, k, plane) : G0T(0);
 #pragma unroll
         for (int p = 0; p < 17; ++p) {
@@ -553,20 +555,18 @@ __global__ void __launch_bounds__(NTMAX, 1) k_resident(const __grid_constant__ R
         if (!own && want) sRing[atomicAdd(&s_n[2], 1)] = (uint16_t)c;
     }
     __syncthreads();
-    if constexpr (!BATCH) {
-        if (q.steps == 0) {                       // only the lists' lengths
-            for (int c = tid; c < area; c += NT) {
-                const int ly = c / rs - kHaloY, lx = c % rs - kHaloX, n = __popc(mask[c]);
-                if (n) atomicAdd(&s_n[lx >= 0 && lx < r.w && ly >= 0 && ly < r.h], n);
-            }
-            __syncthreads();
-            if (tid == 0) {
-                const int poll = s_n[0] + kMostHeartbeats;
-                atomicMax(&q.need[0], (poll > s_n[1] ? poll : s_n[1]) - L::CAP);
-                atomicMax(&q.need[1], s_n[4] - L::COPIES);
-            }
-            return;
+    if constexpr (COUNT) {
+        for (int c = tid; c < area; c += NT) {
+            const int ly = c / rs - kHaloY, lx = c % rs - kHaloX, n = __popc(mask[c]);
+            if (n) atomicAdd(&s_n[lx >= 0 && lx < r.w && ly >= 0 && ly < r.h], n);
         }
+        __syncthreads();
+        if (tid == 0) {
+            const int poll = s_n[0] + kMostHeartbeats;
+            atomicMax(&q.need[0], (poll > s_n[1] ? poll : s_n[1]) - L::CAP);
+            atomicMax(&q.need[1], s_n[4] - L::COPIES);
+        }
+        return;
     }
     for (int p = 0; p < kTypes; ++p) {
         for (int c0 = tid & ~31; c0 < area; c0 += NT) {
@@ -927,7 +927,9 @@ template <int PREC, int VV, int K, bool BATCH>
 cudaError_t launch_k(const ResArgs<PREC, BATCH>& q, int n_items, int nt, cudaStream_t stream)
 {
     constexpr Class c = class_of(PREC, K);
-    auto* k = k_resident<PREC, VV, c.wm, c.hm, c.p, c.nt, BATCH>;
+    auto* k = k_resident<PREC, VV, c.wm, c.hm, c.p, c.nt, BATCH, false>;
+    if constexpr (!BATCH)
+        if (q.steps == 0) k = k_resident<PREC, 0, c.wm, c.hm, c.p, c.nt, false, true>;
     constexpr int smem = Lay<PREC, c.wm, c.hm>::kBytes;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
