@@ -10,9 +10,9 @@
 //
 // Measured (us per step in runs of 1000, one launch per step -> resident; the
 // launches in brackets overlap their heads and tails, launch_after):
-// FP32 100 x 50 6.16 (5.1) -> 1.92, 256 x 128 6.17 (5.8) -> 2.34, 400 x 200 with
-// a 30 degree slope 8.21 (6.6) -> 2.65, 512 x 512 with a disc 10.3 (9.7) -> 5.9
-// (BF16 10.7 (9.9) -> 4.9); FP64 100 x 50 18.4 -> 6.1, 400 x 200 41.0 -> 18.2. What a step of 256 x 128
+// FP32 100 x 50 6.16 (5.1) -> 1.85, 256 x 128 6.17 (5.8) -> 2.29, 400 x 200 with
+// a 30 degree slope 8.21 (6.6) -> 2.62, 512 x 512 with a disc 10.3 (9.7) -> 5.8
+// (BF16 10.7 (9.9) -> 4.8); FP64 100 x 50 18.4 -> 6.1, 400 x 200 41.0 -> 18.2. What a step of 256 x 128
 // takes (cycles, a patch at the wall): bounce-back copies, pulls and phi
 // 1,100, ghost values 800, collision 1,000, publishing 400, the wait 1,650. With
 // larger patches the pulls (shared-memory bandwidth) and the collision (FP32
